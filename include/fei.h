@@ -64,10 +64,13 @@ typedef enum {
 } fei_status;
 
 typedef enum {
-  /* Everything in FP64 on the CUDA cores: the plain FP64 GPU path. */
+  /* Everything in FP64 on the CUDA cores: sum factorisation at degrees
+   * >= 2 (see FEI_SF_FP32), the double loop at degree 1. */
   FEI_FP64 = 0,
-  /* FP64 Jacobian columns and w det J; FP32 point operator, FP32
-   * contraction on the CUDA cores.  Output FP32. */
+  /* Vertex differences in FP64, element vectors and w det J in double-FP32
+   * (rounded once), FP32 point operator and sums on the CUDA cores: sum
+   * factorisation at degrees >= 2, the double loop at degree 1.  Output
+   * FP32. */
   FEI_FP32 = 1,
   /* As FEI_FP32 for the geometry and point operator; the contraction runs
    * on the tcgen05 tensor cores with each operand split into fp16 hi + lo
@@ -82,14 +85,13 @@ typedef enum {
    * bf16's 8 significant bits need three pieces and six products for the
    * same accuracy.  Degrees 1 and 2 fall back to FEI_FP32.  Output FP32. */
   FEI_TC_3XTF32 = 3,
-  /* Sum factorisation on the CUDA cores (degrees >= 3): the basis and the
-   * collapsed rule are tensor products in (u, v, zeta), so each component
-   * of the reference gradient is a sum of one or two products of 1D
-   * factors and the sum over points runs as three short sums, u then v
-   * then zeta, over the 21 pairs of gradient terms (about 7x fewer
-   * multiply-adds than the dense contraction at p = 7).  Geometry and
-   * point operator as FEI_FP32, the sums in FP32.  Degrees 1 and 2 fall
-   * back to FEI_FP32.  Output FP32. */
+  /* Sum factorisation on the CUDA cores: in the collapsed coordinates
+   * (u, v, zeta) the basis, its derivatives and the rule are products of 1D
+   * factors, so the sum over points runs as three short sums, u then v then
+   * zeta, over the 13 pairs of separable gradient terms (24 times fewer
+   * flops than the dense contraction at p = 4, 92 times at p = 7).  The same
+   * kernel as FEI_FP32 at degrees >= 2; degree 1 falls back to FEI_FP32.
+   * Output FP32. */
   FEI_SF_FP32 = 4,
   /* Per degree, the fastest kernel among those measured within 1e-6 of
    * the FP64 oracle (relative Frobenius norm per element): the FEI_FP32

@@ -213,7 +213,7 @@ fei_status launch_forward(int p, fei_precision prec, const fei_reference *r, con
   const KernelKind k = direct_kernel(prec, p, &run);
   const fei_status st = k == KERNEL_TC   ? launch_tc_forward(p, r, a, grid_work, s, 0, run)
                         : k == KERNEL_SF ? launch_sf_forward(p, r, a, grid_work, s)
-                                         : launch_cc_forward(p, run == FEI_FP64, a, grid_work, s);
+                                         : launch_cc_forward(p, run == FEI_FP64, r, a, grid_work, s);
   return st ? st : debug_check(s, "forward kernel");
 }
 

@@ -11,7 +11,7 @@
 //   tnode double [(p+1)^2][4]    (xi1, xi2, w_tri, 0)  collapsed triangle nodes
 //   point q = iz * (p+1)^2 + t, t = iv * (p+1) + iu, w_q = w_tri[t] w_zeta[iz].
 //   tc    the tensor-core B operand images and paired tables (fei_tc.cu).
-//   sf    FP32 1D factor tables of the sum-factorised path (fei_sf.cu).
+//   sf, sf64  1D factor tables of the sum-factorised paths (fei_sf1d.cuh).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -26,6 +26,7 @@ constexpr int kPMax = 7;
 
 __host__ __device__ constexpr int nsh_of(int p) { return (p + 1) * (p + 1) * (p + 2) / 2; }
 __host__ __device__ constexpr int nq_of(int p) { return (p + 1) * (p + 1) * (p + 1); }
+
 __host__ __device__ constexpr int ntri_of(int p) { return (p + 1) * (p + 2) / 2; }
 
 struct TcImage;  // tensor-core operand image, fei_tc.cu
@@ -42,7 +43,8 @@ struct fei_reference {
   double *tnode;
   float *G32T;       // [N_q][N_sh][4] the FP32 table with the 4 components adjacent
   fei::TcImage *tc;  // null until built (degree >= 3)
-  float *sf;         // 1D factor tables of the sum-factorised path (degree >= 3), or null
+  float *sf;         // 1D factor tables of the sum-factorised paths, or null
+  double *sf64;      // the same in FP64
 };
 
 namespace fei {
@@ -145,8 +147,8 @@ fei_status integrate_scratch(const fei_reference *const *by_p, const fei_batch *
 // Kernel launchers (each returns FEI_OK or an error already recorded).
 // grid_cap: largest grid (blocks) of the grid-stride kernels, 0 = default
 // (all work items for a known count, 152 x 4 or 152 x 8 for a device count)
-fei_status launch_cc_forward(int p, bool fp64, const FwdArgs &a, int64_t grid_work, cudaStream_t s,
-                             int64_t grid_cap = 0);
+fei_status launch_cc_forward(int p, bool fp64, const fei_reference *ref, const FwdArgs &a, int64_t grid_work,
+                             cudaStream_t s, int64_t grid_cap = 0);
 // quadratic = true: the adjoint of L = sum_e u_e^T A_e u_e - u_e^T b_e
 // (gA_e = u_e u_e^T and gb_e = -u_e never formed; a.u holds u)
 fei_status launch_cc_backward(int p, bool fp64, const BwdArgs &a, int64_t grid_work, cudaStream_t s,
@@ -172,6 +174,8 @@ inline KernelKind direct_kernel(fei_precision prec, int p, fei_precision *run) {
 }
 fei_status launch_sf_forward(int p, const fei_reference *ref, const FwdArgs &a, int64_t grid_work, cudaStream_t s,
                              int64_t grid_cap = 0);
+fei_status launch_sf64_forward(int p, const fei_reference *ref, const FwdArgs &a, int64_t grid_work, cudaStream_t s,
+                               int64_t grid_cap = 0);
 fei_status build_sf_tables(fei_reference *ref);
 void free_sf_tables(fei_reference *ref);
 // variant: 0 .. tc_variant_count(p, prec) - 1 (warp-role variants of one

@@ -142,7 +142,7 @@ fei_status launch_degree(const fei_plan *pl, int p, int variant, int64_t grid_ca
   const KernelKind k = plan_kernel(pl->prec, p, variant, &run);
   const fei_status ls = k == KERNEL_TC   ? launch_tc_forward(p, r, a, b->n_elem, s, variant, run)
                         : k == KERNEL_SF ? launch_sf_forward(p, r, a, b->n_elem, s, grid_cap)
-                                         : launch_cc_forward(p, run == FEI_FP64, a, b->n_elem, s, grid_cap);
+                                         : launch_cc_forward(p, run == FEI_FP64, r, a, b->n_elem, s, grid_cap);
   return ls ? ls : debug_check(s, "forward kernel");
 }
 

@@ -228,13 +228,11 @@ extern "C" fei_status fei_reference_create(int p, fei_reference_t *out) {
     fei_reference_destroy(r);
     return cuda_error(e, "reference tabulation kernels");
   }
-  if (p >= 3) {
-    fei_status st = build_tc_image(r);
-    if (st == FEI_OK) st = build_sf_tables(r);
-    if (st != FEI_OK) {
-      fei_reference_destroy(r);
-      return st;
-    }
+  fei_status st = p >= 3 ? build_tc_image(r) : FEI_OK;
+  if (st == FEI_OK) st = build_sf_tables(r);
+  if (st != FEI_OK) {
+    fei_reference_destroy(r);
+    return st;
   }
   *out = r;
   return FEI_OK;

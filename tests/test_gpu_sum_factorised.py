@@ -1,0 +1,97 @@
+"""The sum-factorised forward at the sizes where it can go wrong: counts
+around a block's batch of elements (1 to 4), more batches than resident
+blocks (the persistent loop and its record prefetch), a bucketed list, flat
+and tiny elements (w det J formed again in FP64), against the FP64 oracle.
+Tolerances are the paths' own bars."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1310_1194_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+TOL = {"fp64": 1e-12, "fp32": 1e-5, "sf_fp32": 1e-5}
+
+
+def run(w, precision, p=None, degree=None, **kw):
+    from paper_1310_1194_gb300 import api
+    g = [torch.from_numpy(np.ascontiguousarray(w[k])).cuda() for k in ("geom", "K", "b", "c", "f")]
+    d = None if degree is None else torch.from_numpy(np.ascontiguousarray(degree)).to(torch.int32).cuda()
+    A, b, st, _ = api.fei_integrate(*g, p=p, degree=d, precision=precision, **kw)
+    torch.cuda.synchronize()
+    return A.double().cpu().numpy(), b.double().cpu().numpy(), st.cpu().numpy()
+
+
+def per_elem_err(got, want, offsets, sizes):
+    return np.array([np.linalg.norm(got[o:o + k] - want[o:o + k]) / max(np.linalg.norm(want[o:o + k]), 1e-300)
+                     for o, k in zip(offsets, sizes)])
+
+
+def take(w, idx):
+    return {k: np.ascontiguousarray(w[k][idx]) for k in ("geom", "K", "b", "c", "f")}
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("p", range(2, 8))
+def test_counts_around_a_batch(p, precision):
+    """1..5, 7 elements and, on sampled elements, a batch several times the
+    resident blocks: the same element must not depend on its place."""
+    big = {2: 9001, 3: 7001, 4: 5003, 5: 3001, 6: 1201, 7: 701}[p]
+    w = inputs.workload("p4", n_max=big)
+    s = (p + 1) ** 2 * (p + 2) // 2
+    Ab, bb, stb = run(w, precision, p=p)
+    assert not stb.any()
+    idx = np.r_[0:7, big // 2, big - 4:big]
+    ref = oracle.integrate(*(take(w, idx)[k] for k in ("geom", "K", "b", "c", "f")), p=p)
+    off = np.arange(len(idx) + 1)
+    ea = per_elem_err(Ab.reshape(big, -1)[idx].reshape(-1), ref[0], off * s * s, np.full(len(idx), s * s))
+    eb = per_elem_err(bb.reshape(big, -1)[idx].reshape(-1), ref[1], off * s, np.full(len(idx), s))
+    assert ea.max() < TOL[precision] and eb.max() < TOL[precision]
+    for n in (1, 2, 3, 4, 5, 7):
+        A, b, st = run(take(w, np.arange(n)), precision, p=p)
+        assert not st.any()
+        assert np.array_equal(A, Ab[:n * s * s]) and np.array_equal(b, bb[:n * s])
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_bucketed_equals_uniform(precision):
+    """Elements of a list (a degree array) give the uniform call's bits."""
+    w = inputs.workload("pr1", n_max=60)
+    degree = np.tile(np.arange(2, 8, dtype=np.int32), 10)
+    A, b, st = run(w, precision, degree=degree)
+    assert not st.any()
+    s = (degree + 1) ** 2 * (degree + 2) // 2
+    Ao, bo = np.r_[0, np.cumsum(s * s)], np.r_[0, np.cumsum(s)]
+    for e in range(0, 60, 7):
+        Au, bu, _ = run(take(w, [e]), precision, p=int(degree[e]))
+        assert np.array_equal(Au, A[Ao[e]:Ao[e + 1]]) and np.array_equal(bu, b[bo[e]:bo[e + 1]])
+
+
+@pytest.mark.parametrize("p", [2, 3, 4, 6, 7])
+def test_status_of_flat_and_scaled_elements(p):
+    """Mirrored, exactly flat and almost flat elements and meshes scaled to
+    1e-6 and 1e6: the FP32 path's statuses equal the FP64 path's and the
+    oracle's, and unflagged results hold the bar."""
+    w = inputs.workload("pr1", n_max=12)
+    w = {k: w[k].copy() for k in ("geom", "K", "b", "c", "f")}
+    g = w["geom"]
+    g[1] = g[1][[0, 2, 1, 3, 5, 4]]
+    g[3, 3:] = g[3, :3]
+    g[5, 3:] = g[5, :3] + 1e-5 * (g[5, 3:] - g[5, :3])
+    g[7] *= 1e-6
+    g[8] *= 1e6
+    g[10, 2, 1] = np.inf
+    A64, b64, s64 = run(w, "fp64", p=p)
+    A32, b32, s32 = run(w, "fp32", p=p)
+    Ao, bo, so, (Aoff, _, _) = oracle.integrate(w["geom"], w["K"], w["b"], w["c"], w["f"], p=p)
+    assert np.array_equal(s64, so) and np.array_equal(s32, so)
+    assert set(np.flatnonzero(so)) == {1, 3, 10}
+    s = (p + 1) ** 2 * (p + 2) // 2
+    sizes = np.full(12, s * s)
+    keep = so == 0
+    assert per_elem_err(A64, Ao, Aoff, sizes)[keep].max() < 1e-12
+    assert per_elem_err(A32, Ao, Aoff, sizes)[keep].max() < 1e-5
+    assert not A32.reshape(12, -1)[~keep].any() and not b32.reshape(12, -1)[~keep].any()
