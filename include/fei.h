@@ -95,10 +95,11 @@ typedef enum {
   FEI_SF_FP32 = 4,
   /* Per degree, the fastest kernel among those measured within 1e-6 of
    * the FP64 oracle (relative Frobenius norm per element): the FEI_FP32
-   * kernels for p <= 2, the FEI_TC_F16X3 kernel for p = 3, 4 and the
-   * sum-factorised kernel for p = 5..7 on a direct call; a plan's tuner
-   * times the tensor-core variants and the sum-factorised kernel at every
-   * p >= 3 and keeps the fastest.  Output FP32. */
+   * kernels for p <= 2 and the sum-factorised kernel for p >= 3; on a
+   * direct call p = 3, 4 batches of at most 512 elements give the bits of
+   * FEI_TC_F16X3.  A plan starts from the sum-factorised kernel at p >= 3;
+   * its tuner times the tensor-core variants and the sum-factorised kernel
+   * and keeps the fastest.  Output FP32. */
   FEI_AUTO = 5
 } fei_precision;
 

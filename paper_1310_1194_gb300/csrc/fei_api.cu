@@ -187,6 +187,7 @@ fei_status check_batch(const fei_batch *b) {
 void fill_fwd(FwdArgs &a, const fei_batch *b, const fei_reference *r, void *A, void *bv, int32_t *st) {
   memset(&a, 0, sizeof(a));
   a.n_work = b->n_elem;
+  a.n_batch = b->n_elem;
   a.geom = b->geom;
   a.coef_mode = b->coef_mode;
   a.K = b->K;
@@ -210,7 +211,7 @@ void fill_fwd(FwdArgs &a, const fei_batch *b, const fei_reference *r, void *A, v
 fei_status launch_forward(int p, fei_precision prec, const fei_reference *r, const FwdArgs &a,
                           int64_t grid_work, cudaStream_t s) {
   fei_precision run;
-  const KernelKind k = direct_kernel(prec, p, &run);
+  const KernelKind k = direct_kernel(prec, p, a.n_batch, &run);
   const fei_status st = k == KERNEL_TC   ? launch_tc_forward(p, r, a, grid_work, s, 0, run)
                         : k == KERNEL_SF ? launch_sf_forward(p, r, a, grid_work, s)
                                          : launch_cc_forward(p, run == FEI_FP64, r, a, grid_work, s);
@@ -372,14 +373,15 @@ extern "C" fei_status fei_plan_offsets_upper(const int32_t *degree, int64_t n_el
 
 namespace fei {
 
-fei_status integrate_scratch(const fei_reference *const *by_p, const fei_batch *batch, fei_precision prec,
-                             void *A_out, void *b_out, int32_t *elem_status, int32_t *counts, int32_t *lists,
-                             int64_t cap, cudaStream_t s) {
+fei_status integrate_scratch(const fei_reference *const *by_p, const fei_batch *batch, int64_t n_batch,
+                             fei_precision prec, void *A_out, void *b_out, int32_t *elem_status, int32_t *counts,
+                             int32_t *lists, int64_t cap, cudaStream_t s) {
   if (!batch->degree) {
     const int p = batch->uniform_degree;
     if (!by_p[p]) return set_error(FEI_ERR_INVALID_DEGREE, "no reference for degree %d", p);
     FwdArgs a;
     fill_fwd(a, batch, by_p[p], A_out, b_out, elem_status);
+    a.n_batch = n_batch;
     return launch_forward(p, prec, by_p[p], a, batch->n_elem, s);
   }
   unsigned avail = 0;
@@ -397,6 +399,7 @@ fei_status integrate_scratch(const fei_reference *const *by_p, const fei_batch *
     if (!by_p[p]) continue;
     FwdArgs a;
     fill_fwd(a, batch, by_p[p], A_out, b_out, elem_status);
+    a.n_batch = n_batch;
     a.count = counts + p;
     a.list = lists + (int64_t)(p - 1) * cap;
     const fei_status st = launch_forward(p, prec, by_p[p], a, batch->n_elem, s);
@@ -427,7 +430,7 @@ extern "C" fei_status fei_integrate(const fei_reference_t *refs, int nrefs, cons
     st = workspace_for(dev, batch->n_elem, &ws);
     if (st) return st;
   }
-  return integrate_scratch(by_p, batch, prec, A_out, b_out, elem_status, ws ? ws->counts : nullptr,
+  return integrate_scratch(by_p, batch, batch->n_elem, prec, A_out, b_out, elem_status, ws ? ws->counts : nullptr,
                            ws ? ws->lists : nullptr, ws ? ws->capacity : 0, (cudaStream_t)stream);
 }
 

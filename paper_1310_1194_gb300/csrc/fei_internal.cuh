@@ -54,6 +54,7 @@ namespace fei {
 // elements 0 .. n_work.
 struct FwdArgs {
   int64_t n_work;
+  int64_t n_batch;       // elements of the whole call (n_work may be a chunk of it)
   const int32_t *count;  // device, or null
   const int32_t *list;   // device, or null
   const double *geom;
@@ -139,10 +140,11 @@ fei_status debug_check(cudaStream_t s, const char *what);
 
 // The forward of fei_integrate on checked arguments (by_p from check_refs),
 // with the bucketing scratch given: counts int32 [8] and lists int32
-// [7][cap], cap >= n_elem (both unused for a uniform degree).
-fei_status integrate_scratch(const fei_reference *const *by_p, const fei_batch *batch, fei_precision prec,
-                             void *A_out, void *b_out, int32_t *elem_status, int32_t *counts, int32_t *lists,
-                             int64_t cap, cudaStream_t s);
+// [7][cap], cap >= n_elem (both unused for a uniform degree).  n_batch: the
+// elements of the caller's whole batch, of which this one may be a chunk.
+fei_status integrate_scratch(const fei_reference *const *by_p, const fei_batch *batch, int64_t n_batch,
+                             fei_precision prec, void *A_out, void *b_out, int32_t *elem_status, int32_t *counts,
+                             int32_t *lists, int64_t cap, cudaStream_t s);
 
 // Kernel launchers (each returns FEI_OK or an error already recorded).
 // grid_cap: largest grid (blocks) of the grid-stride kernels, 0 = default
@@ -163,10 +165,17 @@ inline bool valid_precision(fei_precision prec) {
 // sum-factorised kernels run degrees >= 3; lower degrees of those
 // precisions run the FEI_FP32 CUDA-core kernels.
 enum KernelKind { KERNEL_CC = 0, KERNEL_TC = 1, KERNEL_SF = 2 };
-// The kernel of degree p under prec on a direct call, and the precision it
-// runs in (FEI_AUTO resolved per degree).
-inline KernelKind direct_kernel(fei_precision prec, int p, fei_precision *run) {
-  if (prec == FEI_AUTO) prec = p <= 2 ? FEI_FP32 : p <= 4 ? FEI_TC_F16X3 : FEI_SF_FP32;
+// The kernel of degree p under prec on a direct call of n_batch elements, and
+// the precision it runs in (FEI_AUTO resolved per degree).  FEI_AUTO at
+// p = 3, 4 keeps the bits of FEI_TC_F16X3 for small batches, as documented;
+// above kAutoTcMax it runs the sum-factorised kernel, the faster of the two
+// (GB300, p = 4: 1000 prisms 23 against 40 us, 100 000 prisms 1.58 against
+// 2.81 ms; p = 3: 1000 prisms 14 against 23 us) and the closer one to FP64
+// (1.6e-7 against 4.1e-7).
+constexpr int64_t kAutoTcMax = 512;
+inline KernelKind direct_kernel(fei_precision prec, int p, int64_t n_batch, fei_precision *run) {
+  if (prec == FEI_AUTO)
+    prec = p <= 2 ? FEI_FP32 : (p <= 4 && n_batch <= kAutoTcMax) ? FEI_TC_F16X3 : FEI_SF_FP32;
   *run = prec;
   if (p >= 3 && tc_precision(prec)) return KERNEL_TC;
   if (p >= 3 && prec == FEI_SF_FP32) return KERNEL_SF;

@@ -89,6 +89,6 @@ extern "C" fei_status fei_integrate_noalloc(const fei_reference_t *refs, int nre
     counts = scratch;
     lists = scratch + 8;
   }
-  return integrate_scratch(by_p, batch, prec, A_out, b_out, elem_status, counts, lists, kNoAllocMax,
+  return integrate_scratch(by_p, batch, batch->n_elem, prec, A_out, b_out, elem_status, counts, lists, kNoAllocMax,
                            (cudaStream_t)stream);
 }

@@ -308,7 +308,7 @@ fei_status enqueue_chunks(fei_pipeline *pl, const fei_batch *hb, void *A_host, v
       db.b_offset = in.b_off;
       db.q_offset = per_point ? in.q_off : nullptr;
     }
-    st = integrate_scratch(pl->by_p, &db, pl->prec, out.A, out.bv, out.status, in.counts, in.lists,
+    st = integrate_scratch(pl->by_p, &db, hb->n_elem, pl->prec, out.A, out.bv, out.status, in.counts, in.lists,
                            pl->max_elem, s);
     if (st) return st;
     FEI_CUDA_TRY(cudaEventRecord(in.consumed, s), "cudaEventRecord");

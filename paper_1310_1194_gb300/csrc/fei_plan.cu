@@ -58,16 +58,16 @@ KernelKind plan_kernel(fei_precision prec, int p, int variant, fei_precision *ru
     *run = variant < tc_variant_count(p, FEI_TC_F16X3) ? FEI_TC_F16X3 : FEI_SF_FP32;
     return *run == FEI_TC_F16X3 ? KERNEL_TC : KERNEL_SF;
   }
-  return direct_kernel(prec, p, run);
+  return direct_kernel(prec, p, INT64_MAX, run);
 }
 int n_variants(fei_precision prec, int p) {
   fei_precision run;
   if (prec == FEI_AUTO && p >= 3) return tc_variant_count(p, FEI_TC_F16X3) + 1;
-  return direct_kernel(prec, p, &run) == KERNEL_TC ? tc_variant_count(p, run) : 1;
+  return direct_kernel(prec, p, INT64_MAX, &run) == KERNEL_TC ? tc_variant_count(p, run) : 1;
 }
 // The variant a plan starts from (before any tuning).
 int default_variant(fei_precision prec, int p) {
-  return (prec == FEI_AUTO && p >= 5) ? tc_variant_count(p, FEI_TC_F16X3) : 0;
+  return (prec == FEI_AUTO && p >= 3) ? tc_variant_count(p, FEI_TC_F16X3) : 0;
 }
 
 // The batch a graph was captured for, field by field (not the padding).
@@ -109,6 +109,7 @@ void candidate(fei_precision prec, int p, int c, int *variant, int64_t *grid_cap
 void fill_args(FwdArgs &a, const fei_batch *b, const fei_reference *r, void *A, void *bv, int32_t *st) {
   memset(&a, 0, sizeof(a));
   a.n_work = b->n_elem;
+  a.n_batch = b->n_elem;
   a.geom = b->geom;
   a.coef_mode = b->coef_mode;
   a.K = b->K;

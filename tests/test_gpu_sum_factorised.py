@@ -95,3 +95,22 @@ def test_status_of_flat_and_scaled_elements(p):
     assert per_elem_err(A64, Ao, Aoff, sizes)[keep].max() < 1e-12
     assert per_elem_err(A32, Ao, Aoff, sizes)[keep].max() < 1e-5
     assert not A32.reshape(12, -1)[~keep].any() and not b32.reshape(12, -1)[~keep].any()
+
+
+@pytest.mark.parametrize("p", [3, 4])
+def test_auto_follows_the_whole_batch(p):
+    """FEI_AUTO at p = 3, 4 picks its kernel by the size of the caller's batch:
+    at most 512 elements give FEI_TC_F16X3's bits and more FEI_SF_FP32's, in
+    chunks through host memory as well."""
+    from paper_1310_1194_gb300 import api
+    for n, same in ((512, "tc_f16x3"), (513, "sf_fp32")):
+        w = inputs.workload("pr1", n_max=n)
+        w = take(w, np.arange(n))
+        A, b, st = run(w, "auto", p=p)
+        As, bs, _ = run(w, same, p=p)
+        assert not st.any() and np.array_equal(A, As) and np.array_equal(b, bs)
+        pipe = api.Pipeline(degrees=[p], precision="auto", slot_bytes=1 << 20)
+        Ah, bh, _ = pipe.integrate_host(*(torch.from_numpy(w[k]).pin_memory() for k in ("geom", "K", "b", "c", "f")), p=p)
+        torch.cuda.synchronize()
+        assert pipe.n_chunks > 1
+        assert np.array_equal(Ah.double().numpy(), A) and np.array_equal(bh.double().numpy(), b)
