@@ -216,16 +216,12 @@ fei_status fei_integrate(const fei_reference_t *refs, int nrefs,
  * vertex coordinates g_geom [n_elem][6][3] (FP64) and the coefficients
  * (g_coef, same layout and mode as the inputs, FP64).  Per-point
  * coefficient values are held fixed when differentiating by the geometry.
- * Jacobians are recomputed, not stored.  Precision: FEI_FP64 (all FP64);
- * FEI_FP32 (the contraction W = gA G^T in FP32 on the CUDA cores, the chain
- * in FP32 with det J from FP64 node sums); FEI_TC_F16X3 or FEI_AUTO with a
- * uniform degree 3..5: dL/dDt_q = G_q gA G_q^T with W^T = G gA^T on the
- * tensor cores (each gA row split into fp16 hi + lo with its own
- * power-of-two scale, three products per K slice) and the FP32 chain, in
- * chunks of 8192 elements (FEI_ADJOINT_CHUNK in the environment overrides
- * it) with 64 N_q bytes of scratch per element allocated stream-ordered on
- * the stream; every other precision and case runs as FEI_FP32.  gA and gb
- * are FP32 for every precision but FEI_FP64.
+ * Jacobians are recomputed, not stored.  The contraction is the transpose of
+ * the sum-factorised forward (see FEI_SF_FP32) at every degree.  Precision:
+ * FEI_FP64 (all FP64); every other precision runs the FP32 adjoint (FP32
+ * sums and chain, w det J and det J in double-FP32 rounded once, the sums
+ * over points as FP32 pairs), with gA and gb in FP32.  No scratch memory but
+ * the bucketing workspace of a degree array.
  * Elements with a nonzero elem_status from the forward get zero gradients
  * (this call recomputes the status itself).  batch->a_layout must be
  * FEI_A_FULL (FEI_ERR_UNSUPPORTED otherwise). */
@@ -238,13 +234,12 @@ fei_status fei_integrate_backward(const fei_reference_t *refs, int nrefs,
 /* Adjoint of the quadratic loss L = sum_e u_e^T A_e u_e - u_e^T b_e (the
  * energy of a field u; not in the paper): the gradients fei_integrate_backward
  * gives for gA_e = u_e u_e^T and gb_e = -u_e, computed without forming gA.
- * With v_q = G_q u_e (value and reference gradient of the field at point q),
- * dL/dDt_q = v_q v_q^T and dL/d(w det J f)_q = -v_q[0], so the cost per
- * element is O(N_sh N_q) instead of O(N_sh^2 N_q).
+ * With v_q = G_q u_e (value and reference gradient of the field at point q,
+ * by three one-dimensional sums), dL/dDt_q = v_q v_q^T and
+ * dL/d(w det J f)_q = -v_q[0], so the cost per element is the chain's.
  *  u  device double [b_total]: u_e at b_offset[e] (the layout of b_out).
  * Other arguments, outputs, precisions and errors as for
- * fei_integrate_backward (FEI_FP32: v_q in FP32, the Jacobian chain in
- * FP64). */
+ * fei_integrate_backward. */
 fei_status fei_integrate_backward_quadratic(const fei_reference_t *refs, int nrefs,
                                             const fei_batch *batch, fei_precision prec,
                                             const double *u, double *g_geom,

@@ -244,10 +244,8 @@ def fei_integrate_backward(geom, K, b, c, f, gA, gb, p=None, degree=None, per_qp
                            precision="fp64", refs=None, layout=None):
     """Gradients of <gA, A> + <gb, b>: (g_geom, gK, gb_coef, gc, gf), FP64.
 
-    precision: "fp64" (gA, gb FP64; all FP64), "fp32" (gA, gb FP32; the FP32
-    adjoint), "tc_f16x3" or "auto" (gA, gb FP32; at a uniform degree 3..5
-    dL/dDt is formed on the tensor cores, elsewhere the FP32 adjoint runs);
-    other split precisions run the FP32 adjoint."""
+    precision: "fp64" (gA, gb FP64; all FP64); every other precision runs the
+    FP32 adjoint (gA, gb FP32)."""
     geom, layout = _inputs(geom, K, b, c, f, degree, p, per_qp, layout)
     prec = _lib.PRECISIONS[precision]
     dtype = torch.float64 if prec == _lib.FEI_FP64 else torch.float32
@@ -599,9 +597,7 @@ class _IntegrateFn(torch.autograd.Function):
     def backward(ctx, gA, gb, _gst):
         geom, K, bc, c, f = ctx.saved_tensors
         p, degree, per_qp, precision, layout = ctx.cfg
-        # the tensor-core adjoint where the forward ran the split fp16 path
-        # (the library runs it at a uniform degree 3..5, else the FP32 one)
-        bprec = "fp64" if precision == "fp64" else "tc_f16x3" if precision in ("tc_f16x3", "auto") else "fp32"
+        bprec = "fp64" if precision == "fp64" else "fp32"
         dt = torch.float64 if bprec == "fp64" else torch.float32
         gA = torch.zeros(layout.A_total, dtype=dt, device=geom.device) if gA is None else gA.to(dt).contiguous()
         gb = torch.zeros(layout.b_total, dtype=dt, device=geom.device) if gb is None else gb.to(dt).contiguous()

@@ -164,7 +164,7 @@ __host__ __device__ inline float2 split_f64_bits(double x, bool *in_range) {
 }
 // FP64 -> FP32 rounded to nearest (ties to even) from the bit fields, for
 // a finite x whose FP32 result is normal or overflows; other magnitudes
-// take the conversion instruction (which runs on the FP64 pipe).
+// take the conversion instruction.
 __host__ __device__ inline float f64_to_f32_bits(double x) {
   unsigned long long b;
   memcpy(&b, &x, 8);

@@ -107,14 +107,8 @@ struct BwdArgs {
   const void *gA;
   const void *gb;
   const double *u;  // quadratic-loss adjoint: u_e at b_off[e] (else unused)
-  // general adjoint with dL/dDt precomputed (FEI_FP32 chain only): gDpre
-  // [n_work][N_q][16] for the work items, element e0 + item (no list)
-  const float *gDpre;
-  int64_t e0;
   double *g_geom;
   double *gK, *gbc, *gc, *gf;
-  const double *G64;
-  const float *G32;
   const double *znode;
   const double *tnode;
 };
@@ -153,8 +147,8 @@ fei_status launch_cc_forward(int p, bool fp64, const fei_reference *ref, const F
                              cudaStream_t s, int64_t grid_cap = 0);
 // quadratic = true: the adjoint of L = sum_e u_e^T A_e u_e - u_e^T b_e
 // (gA_e = u_e u_e^T and gb_e = -u_e never formed; a.u holds u)
-fei_status launch_cc_backward(int p, bool fp64, const BwdArgs &a, int64_t grid_work, cudaStream_t s,
-                              bool quadratic = false);
+fei_status launch_cc_backward(int p, bool fp64, const fei_reference *ref, const BwdArgs &a, int64_t grid_work,
+                              cudaStream_t s, bool quadratic = false);
 // The tensor-core precisions (split fp16 or split TF32 operands).
 inline bool tc_precision(fei_precision prec) { return prec == FEI_TC_F16X3 || prec == FEI_TC_3XTF32; }
 inline bool valid_precision(fei_precision prec) {
@@ -192,12 +186,6 @@ void free_sf_tables(fei_reference *ref);
 fei_status launch_tc_forward(int p, const fei_reference *ref, const FwdArgs &a, int64_t grid_work,
                              cudaStream_t s, int variant, fei_precision prec);
 int tc_variant_count(int p, fei_precision prec);
-// Tensor-core adjoint (fei_tc.cu, p = 3..5, uniform degree): gD [count][N_q]
-// [16] = dL/dDt_q of the elements e0 .. e0 + count - 1, from gA (FP32, at
-// A_off[e] or e N_sh^2) with W^T = G gA^T on the tensor cores (split fp16).
-bool tc_adjoint_ready(const fei_reference *ref);  // degree 3..5 and its image built
-fei_status launch_tc_adjoint(int p, const fei_reference *ref, const float *gA, const int64_t *A_off, int64_t e0,
-                             int64_t count, float *gD, cudaStream_t s);
 fei_status build_tc_image(fei_reference *ref);
 void free_tc_image(fei_reference *ref);
 

@@ -143,8 +143,8 @@ __global__ void pack_tables_kernel(int p, const double *t64, const double *znode
   const int M = p + 1, NT = M * (M + 1) / 2;
   const double *U = t64, *V = U + 3 * M * M, *Z = V + 4 * M * NT;
   // SfTab's offsets for a run-time degree
-  const int o_u0 = 2 * M * 4, o_vc = o_u0 + (M * M + 3) / 4 * 4, o_vr = o_vc + (2 * M * NT + 3) / 4 * 4,
-            o_zl = o_vr + (2 * M * NT + 3) / 4 * 4, o_gv = o_zl + M * M, o_su = o_gv + M, o_mt = o_su + M;
+  const int o_u0 = 2 * M * 4, o_u1 = o_u0 + (M * M + 3) / 4 * 4, o_vc = o_u1 + (M * M + 3) / 4 * 4, o_vr = o_vc + (2 * M * NT + 3) / 4 * 4,
+            o_zl = o_vr + (2 * M * NT + 3) / 4 * 4, o_zd = o_zl + M * M, o_gv = o_zd + M * M, o_su = o_gv + M, o_mt = o_su + M;
   const int stride = gridDim.x * blockDim.x, i0 = blockIdx.x * blockDim.x + threadIdx.x;
   for (int i = i0; i < 2 * M * 4; i += stride) {
     const int kind = i / (M * 4), m = i / 4 % M, iu = i % 4;
@@ -152,7 +152,9 @@ __global__ void pack_tables_kernel(int p, const double *t64, const double *znode
   }
   for (int i = i0; i < M * M; i += stride) {
     out[o_u0 + i] = (T)U[(i % M) * M + i / M];
+    out[o_u1 + i] = (T)U[(M + i % M) * M + i / M];
     out[o_zl + i] = (T)Z[(i % M) * M + i / M];
+    out[o_zd + i] = (T)Z[(M + i % M) * M + i / M];
   }
   for (int i = i0; i < M * NT; i += stride) {
     const int iv = i / NT, t = i % NT;

@@ -42,7 +42,7 @@
 #include "fei_elem32.cuh"
 #include "fei_geom.cuh"
 #include "fei_internal.cuh"
-#include "fei_sf1d.cuh"
+#include "fei_sf_ops.cuh"
 
 namespace fei {
 
@@ -112,13 +112,7 @@ struct SfCfg {
   static_assert(E <= NW, "one warp per element in the setup");
 };
 
-// Element data of one slot.  FP64: node columns and the coefficients.
-template <int P>
-struct Elem64 {
-  static constexpr int M = P + 1;
-  double X[18];
-  double zc1[M][3], zc2[M][3], zn3[M][3], tc3[M * M][3];
-};
+// Element data of one slot.
 template <typename T, int P>
 struct SfElem {
   std::conditional_t<std::is_same<T, float>::value, Elem32<P>, Elem64<P>> el;
@@ -126,94 +120,10 @@ struct SfElem {
   T cf[14];
   int status;
 };
-template <int P>
-struct SfNodes64 {
-  double zz[P + 1], zw[P + 1], tx[(P + 1) * (P + 1)][2], tw[(P + 1) * (P + 1)];
-};
-
-// Operators in shared memory: [op][iv][l][iu], the M values of a u row
-// without a pad.  Rows of one quarter-warp fall in distinct banks for M = 4, 6
-// (16- and 8-byte loads) and odd M (4-byte loads); for M = 8 the 16-byte
-// halves are swapped by bit 2 of l, and iv has a stride of 72, so that the
-// columns of the zeta transform are free of conflicts too.
-template <typename T, int M>
-struct OpPos {
-  static constexpr bool SWZ = std::is_same<T, float>::value && M == 8;
-  static constexpr int IV = SWZ ? 72 : M * M, OP = M * IV;
-  static __device__ __forceinline__ int row(int op, int iv, int l) { return op * OP + iv * IV + l * M; }
-  static __device__ __forceinline__ int at(int op, int iv, int l, int iu) {
-    return row(op, iv, l) + (SWZ ? iu ^ (l & 4) : iu);
-  }
-};
-// the u row of (op, iv, l); sw = l & 4 for the swapped halves
-template <int M>
-__device__ __forceinline__ void load_u_row(const float *D, int sw, float *d) {
-  if constexpr (M == 8) {
-    const float4 v = *reinterpret_cast<const float4 *>(D + sw), w = *reinterpret_cast<const float4 *>(D + (sw ^ 4));
-    d[0] = v.x, d[1] = v.y, d[2] = v.z, d[3] = v.w, d[4] = w.x, d[5] = w.y, d[6] = w.z, d[7] = w.w;
-  } else if constexpr (M == 4) {
-    const float4 v = *reinterpret_cast<const float4 *>(D);
-    d[0] = v.x, d[1] = v.y, d[2] = v.z, d[3] = v.w;
-  } else if constexpr (M % 2 == 0) {
-#pragma unroll
-    for (int c = 0; c < M / 2; ++c) {
-      const float2 v = reinterpret_cast<const float2 *>(D)[c];
-      d[2 * c] = v.x, d[2 * c + 1] = v.y;
-    }
-  } else {
-#pragma unroll
-    for (int c = 0; c < M; ++c) d[c] = D[c];
-  }
-}
-template <int M>
-__device__ __forceinline__ void load_u_row(const double *D, int, double *d) {
-#pragma unroll
-  for (int c = 0; c < M; ++c) d[c] = D[c];
-}
-// N values from a 16-byte aligned address (the pad after them may be read)
-template <int N>
-__device__ __forceinline__ void load_vec(const float *s, float *d) {
-  if constexpr (N > 2) {
-    const float4 v = *reinterpret_cast<const float4 *>(s);
-    d[0] = v.x, d[1] = v.y, d[2] = v.z;
-    if constexpr (N > 3) d[3] = v.w;
-  } else if constexpr (N == 2) {
-    const float2 v = *reinterpret_cast<const float2 *>(s);
-    d[0] = v.x, d[1] = v.y;
-  } else {
-    d[0] = s[0];
-  }
-}
-template <int N>
-__device__ __forceinline__ void load_vec(const double *s, double *d) {
-#pragma unroll
-  for (int i = 0; i < N; i += 2) {
-    if (i + 1 < N) {
-      const double2 v = *reinterpret_cast<const double2 *>(s + i);
-      d[i] = v.x, d[i + 1] = v.y;
-    } else {
-      d[i] = s[i];
-    }
-  }
-}
-template <typename T>
-struct Vec2;
-template <> struct Vec2<float> { using type = float2; };
-template <> struct Vec2<double> { using type = double2; };
-
 // Stage 4: the X values of one (iv, l) for the row functions m = g and
 // m = M-1-g and every m', x[j][m'] += sum_iu U_UA(m, iu) U_UB(m', iu) d[iu].
 // The factors are even or odd in u, so the sum runs over half the nodes on
 // e = d(u) + d(-u) or o = d(u) - d(-u).
-template <typename T, int M>
-__device__ __forceinline__ void even_odd(const T *d, T *e, T *o) {
-#pragma unroll
-  for (int i = 0; i < (M + 1) / 2; ++i) {
-    const bool mid = 2 * i == M - 1;
-    e[i] = mid ? d[i] : d[i] + d[M - 1 - i];
-    o[i] = mid ? T(0) : d[i] - d[M - 1 - i];
-  }
-}
 // p <= 5: the products of the two factors are constants of the code
 template <typename T, int P, int G, int UA, int UB>
 __device__ __forceinline__ void u_sum_const(const T *e, const T *o, T (*x)[P + 1]) {

@@ -148,19 +148,21 @@ constexpr int kOps = 13;  // point operators Dt00, Dt01..03, Dt11..33
 // nodes, NT triangle functions, half nodes i < (M+1)/2 (the factors of u are
 // even or odd, so the other half of the nodes follows by symmetry):
 //   UH[2][M m][4 iu]   U_kind(m) at the half nodes (zero-padded)
-//   U0[M m][M iu]      A_m at every node (load vector)
+//   U0[M m][M iu], U1  A_m and A_m' at every node
 //   VC[M iv][NT t][2]  B, 2 B' by triangle function
 //   VR[M iv][NT r][2]  the same in row order (m ascending, then n)
-//   ZL[M iz][M k]      L_k (load vector)
+//   ZL[M iz][M k], ZD  L_k and L_k'
 //   GV[M iv]           g = 4 / (1-v)
 //   SU[M iu]           s = (1+u) / 2
 //   MT[NT]             m of t
 template <int P>
 struct SfTab {
   static constexpr int M = P + 1, NT = M * (M + 1) / 2;
-  static constexpr int O_UH = 0, O_U0 = O_UH + 2 * M * 4, O_VC = O_U0 + (M * M + 3) / 4 * 4,
+  static constexpr int O_UH = 0, O_U0 = O_UH + 2 * M * 4, O_U1 = O_U0 + (M * M + 3) / 4 * 4,
+                       O_VC = O_U1 + (M * M + 3) / 4 * 4,
                        O_VR = O_VC + (2 * M * NT + 3) / 4 * 4, O_ZL = O_VR + (2 * M * NT + 3) / 4 * 4,
-                       O_GV = O_ZL + M * M, O_SU = O_GV + M, O_MT = O_SU + M;
+                       O_ZD = O_ZL + M * M,
+                       O_GV = O_ZD + M * M, O_SU = O_GV + M, O_MT = O_SU + M;
   static constexpr int SIZE = (O_MT + NT + 3) / 4 * 4;
 };
 // Index of the triangle function (m, n): total degree ascending, then n; and

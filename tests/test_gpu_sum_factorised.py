@@ -114,3 +114,49 @@ def test_auto_follows_the_whole_batch(p):
         torch.cuda.synchronize()
         assert pipe.n_chunks > 1
         assert np.array_equal(Ah.double().numpy(), A) and np.array_equal(bh.double().numpy(), b)
+
+
+@pytest.mark.parametrize("precision,tol_elem,tol_rec", [("fp64", 1e-10, 1e-10), ("fp32", 1e-6, 1e-5)])
+@pytest.mark.parametrize("p", range(1, 8))
+def test_adjoint_counts_and_lists(p, precision, tol_elem, tol_rec):
+    """The general and the quadratic-loss adjoint on more elements than
+    resident blocks (the persistent loop reuses every buffer): sampled
+    elements against the oracle; single elements, and elements of a list
+    among other degrees, give the same bits."""
+    from paper_1310_1194_gb300 import api
+    from parity_util import assert_grads_close
+    n = {1: 8001, 2: 8001, 3: 5001, 4: 2501, 5: 1601, 6: 901, 7: 701}[p]
+    w = inputs.workload("p4", n_max=n)
+    s = (p + 1) ** 2 * (p + 2) // 2
+    dt = torch.float64 if precision == "fp64" else torch.float32
+    rng = np.random.default_rng(p)
+    gA, gb, u = (torch.from_numpy(rng.standard_normal(m)).cuda() for m in (n * s * s, n * s, n * s))
+    gA, gb = gA.to(dt), gb.to(dt)
+    dev = lambda ww: [torch.from_numpy(np.ascontiguousarray(ww[k])).cuda() for k in ("geom", "K", "b", "c", "f")]  # noqa: E731
+    g = dev(w)
+    full = api.fei_integrate_backward(*g, gA, gb, p=p, precision=precision)
+    quad = api.fei_integrate_backward_quadratic(*g, u, p=p, precision=precision)
+    idx = np.r_[0, 1, n // 2, n - 2, n - 1]
+    sub = take(w, idx)
+    Ai, bi = gA.view(n, -1)[idx].contiguous(), gb.view(n, -1)[idx].contiguous()
+    ui = u.view(n, -1)[idx].cpu().numpy()
+    args = [sub[k] for k in ("geom", "K", "b", "c", "f")]
+    ref = oracle.integrate_backward(*args, Ai.double().cpu().numpy().reshape(-1), bi.double().cpu().numpy().reshape(-1), p=p)
+    nq = np.full(len(idx), (p + 1) ** 3)
+    assert_grads_close([t[idx].cpu().numpy() for t in full], ref, len(idx), False, nq, tol_elem, tol_rec, where=f"general p={p}")
+    uu = np.einsum("ni,nj->nij", ui, ui)
+    ref = oracle.integrate_backward(*args, uu.reshape(-1), -ui.reshape(-1), p=p)
+    assert_grads_close([t[idx].cpu().numpy() for t in quad], ref, len(idx), False, nq, tol_elem, tol_rec, where=f"quad p={p}")
+    # a list of the same elements between elements of another degree
+    other = 1 + p % 7
+    so = (other + 1) ** 2 * (other + 2) // 2
+    degree = torch.tensor([p, other] * len(idx), dtype=torch.int32, device="cuda")
+    mixed = dev({k: np.repeat(sub[k], 2, axis=0) for k in sub})
+    pad = lambda t, m: torch.cat([t, torch.zeros(len(idx), m, dtype=t.dtype, device="cuda")], 1).reshape(-1).contiguous()  # noqa: E731
+    got = api.fei_integrate_backward(*mixed, pad(Ai, so * so), pad(bi, so), degree=degree, precision=precision)
+    for x, y in zip(got, full):
+        assert torch.equal(x[::2], y[idx])
+    one = api.fei_integrate_backward(*(t[2:3].contiguous() for t in dev(sub)), Ai[2].contiguous(), bi[2].contiguous(), p=p,
+                                     precision=precision)
+    for x, y in zip(one, full):
+        assert torch.equal(x[0], y[idx[2]])
