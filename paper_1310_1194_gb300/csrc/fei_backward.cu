@@ -80,28 +80,23 @@ __device__ __forceinline__ int point_status_f(float s) {
   return 0;
 }
 
-__device__ __forceinline__ bool load_coef_b(const BwdArgs &a, int64_t r, double *cd) {
-  bool ok = true;
+// The coefficient record r as T; false if a value is not finite.
+template <typename T>
+__device__ __forceinline__ bool load_coef_b(const BwdArgs &a, int64_t r, T *cf) {
+  double cd[14];
 #pragma unroll
   for (int k = 0; k < 9; ++k) cd[k] = a.K[9 * r + k];
 #pragma unroll
   for (int k = 0; k < 3; ++k) cd[9 + k] = a.b[3 * r + k];
   cd[12] = a.c[r];
   cd[13] = a.f[r];
+  if constexpr (std::is_same<T, float>::value) return coef_to_f32<14>(cd, cf);
+  bool ok = true;
 #pragma unroll
-  for (int k = 0; k < 14; ++k) ok &= finite64(cd[k]);
+  for (int k = 0; k < 14; ++k) ok &= finite64(cf[k] = cd[k]);
   return ok;
 }
 
-// An FP32 value as FP64, exactly, by moving its fields (normal numbers and
-// zero; subnormals, infinities and NaN through the conversion instruction):
-// integer work instead of this part's slow FP64 pipe.
-__device__ __forceinline__ double f32_to_f64(float x) {
-  const uint32_t u = __float_as_uint(x), ex = (u >> 23) & 0xffu;
-  if (ex == 0u || ex == 0xffu) return (double)x;
-  const uint32_t hi = (u & 0x80000000u) | ((ex + 896u) << 20) | ((u & 0x7fffffu) >> 3);
-  return __hiloint2double((int)hi, (int)((u & 7u) << 29));
-}
 // (s, e) with s + e = a + b exactly (Knuth's two-sum), FP32.
 __device__ __forceinline__ float2 two_sum_f(float a, float b) {
   const float s = a + b, bb = s - a;
@@ -129,7 +124,7 @@ struct Pair32 {
   static __device__ __forceinline__ float2 shfl(float2 v, int off) {
     return make_float2(__shfl_xor_sync(0xffffffffu, v.x, off), __shfl_xor_sync(0xffffffffu, v.y, off));
   }
-  static __device__ __forceinline__ double value(float2 v) { return f32_to_f64(v.x) + f32_to_f64(v.y); }
+  static __device__ __forceinline__ double value(float2 v) { return (double)v.x + (double)v.y; }
 };
 struct Plain64 {
   using type = double;
@@ -477,6 +472,17 @@ __global__ void __launch_bounds__(AdjCfg<T, P>::NTH, AdjCfg<T, P>::MINB) backwar
   const T *gAg = reinterpret_cast<const T *>(a.gA), *gbg = reinterpret_cast<const T *>(a.gb);
   const int64_t items = a.count ? (int64_t)(*a.count) : a.n_work;
   const bool perq = a.coef_mode == FEI_COEF_PER_POINT;
+  // this lane's share of an element's record (last warp): a vertex coordinate
+  // or a per-element coefficient
+  auto fetch = [&](int64_t it) -> double {
+    if (warp != NW - 1 || it >= items) return 0.0;
+    const int64_t e = a.list ? (int64_t)a.list[it] : it;
+    if (lane < 18) return a.geom[18 * e + lane];
+    if (perq) return 0.0;
+    const int j = lane - 18;
+    return j < 9 ? a.K[9 * e + j] : j < 12 ? a.b[3 * e + j - 9] : j == 12 ? a.c[e] : a.f[e];
+  };
+  double rec = fetch(blockIdx.x);
   __syncthreads();
 
   for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
@@ -484,15 +490,23 @@ __global__ void __launch_bounds__(AdjCfg<T, P>::NTH, AdjCfg<T, P>::MINB) backwar
     const int64_t aoff = a.A_off ? a.A_off[e] : e * (int64_t)(NSH * NSH);
     const int64_t boff = a.b_off ? a.b_off[e] : e * (int64_t)NSH;
     const int64_t qoff = a.q_off ? a.q_off[e] : e * (int64_t)NQ;
-    // the element's record and node data, by the last warp beside the first sums
-    if (warp == NW - 1) {
-      double rec = 0.0;
-      if (lane < 18) {
-        rec = a.geom[18 * e + lane];
-      } else if (!perq) {
-        const int j = lane - 18;
-        rec = j < 9 ? a.K[9 * e + j] : j < 12 ? a.b[3 * e + j - 9] : j == 12 ? a.c[e] : a.f[e];
+    // the next element's inputs on their way to the L2 (at p = 7 the gA of
+    // all blocks' next elements would fill it)
+    if (item + gridDim.x < items) {
+      const int64_t it = item + gridDim.x, en = a.list ? (int64_t)a.list[it] : it;
+      if (!Q && P <= 6)
+        prefetch_l2(gAg + (a.A_off ? a.A_off[en] : en * (int64_t)(NSH * NSH)), (int)sizeof(T) * NSH * NSH, tid, NTH);
+      if (perq) {
+        const int64_t r = a.q_off ? a.q_off[en] : en * (int64_t)NQ;
+        prefetch_l2(a.K + 9 * r, 72 * NQ, tid, NTH);
+        prefetch_l2(a.b + 3 * r, 24 * NQ, tid, NTH);
+        prefetch_l2(a.c + r, 8 * NQ, tid, NTH);
+        prefetch_l2(a.f + r, 8 * NQ, tid, NTH);
       }
+    }
+    // the element's record (fetched one element ahead) and node data, by the
+    // last warp beside the first sums
+    if (warp == NW - 1) {
       const bool bad = __any_sync(0xffffffffu, !finite64(rec));
       if (lane < 18) {
         E.el.X[lane] = rec;
@@ -515,6 +529,7 @@ __global__ void __launch_bounds__(AdjCfg<T, P>::NTH, AdjCfg<T, P>::MINB) backwar
           else t_column_from_vertices(E.el.X, nodes.tx[i - M][0], nodes.tx[i - M][1], E.el.tc3[i - M]);
         }
       }
+      rec = fetch(item + gridDim.x);
     }
     if constexpr (!Q) {
 #pragma unroll 1
@@ -727,13 +742,7 @@ __global__ void __launch_bounds__(AdjCfg<T, P>::NTH, AdjCfg<T, P>::MINB) backwar
       const int iz = q / NT2, t = q - iz * NT2, iv = t / M, iu = t - iv * M;
       T cf[14];
       if (perq) {
-        double cq[14];
-        if (!load_coef_b(a, qoff + q, cq)) pst = FEI_ERR_NONFINITE;
-#pragma unroll
-        for (int k = 0; k < 14; ++k) {
-          if constexpr (F32) cf[k] = f64_to_f32_bits(cq[k]);
-          else cf[k] = cq[k];
-        }
+        if (!load_coef_b<T>(a, qoff + q, cf)) pst = FEI_ERR_NONFINITE;
       } else {
 #pragma unroll
         for (int k = 0; k < 14; ++k) cf[k] = E.cf[k];
@@ -826,18 +835,12 @@ __global__ void __launch_bounds__(AdjCfg<T, P>::NTH, AdjCfg<T, P>::MINB) backwar
       chain_point<T>(w, s, det, adj, cx1, cx2, cx3, cf, gD00, gD0, gDm, gs, gco, gc1, gc2, gc3);
       if (perq) {
         const int64_t r = qoff + q;
-        double go[14];
 #pragma unroll
-        for (int k = 0; k < 14; ++k) {
-          if constexpr (F32) go[k] = f32_to_f64(gco[k]);
-          else go[k] = gco[k];
-        }
+        for (int k = 0; k < 9; ++k) a.gK[9 * r + k] = gco[k];
 #pragma unroll
-        for (int k = 0; k < 9; ++k) a.gK[9 * r + k] = go[k];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) a.gbc[3 * r + k] = go[9 + k];
-        a.gc[r] = go[12];
-        a.gf[r] = go[13];
+        for (int k = 0; k < 3; ++k) a.gbc[3 * r + k] = gco[9 + k];
+        a.gc[r] = gco[12];
+        a.gf[r] = gco[13];
       } else {
 #pragma unroll
         for (int k = 0; k < 14; ++k) acc[21 + k] += gco[k];
@@ -890,7 +893,7 @@ __global__ void __launch_bounds__(AdjCfg<T, P>::NTH, AdjCfg<T, P>::MINB) backwar
             v = add_pair_f(v, b == 1u ? g : make_float2(-g.x, -g.y));
           }
         }
-        val = 0.5 * (f32_to_f64(v.x) + f32_to_f64(v.y));
+        val = 0.5 * ((double)v.x + (double)v.y);
       } else {
         double v = 0.0;
 #pragma unroll

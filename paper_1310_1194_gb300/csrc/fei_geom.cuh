@@ -178,6 +178,41 @@ __host__ __device__ inline float f64_to_f32_bits(double x) {
   memcpy(&f, &r, 4);
   return f;
 }
+// The N coefficient values x rounded to FP32 (nearest, ties to even) with
+// integer instructions; false if one is not finite.  Zeros and values whose
+// FP32 result is normal (or overflows by rounding up) take the fast path; if
+// any value is outside it, all N take the conversion instruction, which runs
+// on the FP64 pipe (16 cycles a warp) and is volatile here so that the
+// compiler does not execute it ahead of the branch.
+template <int N>
+__device__ __forceinline__ bool coef_to_f32(const double *x, float *f) {
+  bool bad = false;
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    const unsigned h = (unsigned)__double2hiint(x[k]), l = (unsigned)__double2loint(x[k]);
+    // sign and exponent shifted out: low 9 exponent bits and 23 bits of the
+    // significand, the exponent rebiased (1023 -> 127 modulo 512)
+    unsigned t = __funnelshift_l(l, h, 3) + 0x40000000u;
+    t += ((l & 0x1fffffffu) + 0x0fffffffu + (t & 1u)) >> 29;
+    const bool zero = ((h & 0x7fffffffu) | l) == 0u;
+    f[k] = __uint_as_float(zero ? h : (t & 0x7fffffffu) | (h & 0x80000000u));
+    bad |= !zero && ((h >> 20) & 0x7ffu) - 897u > 253u;
+  }
+  bool finite = true;
+  if (bad) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      finite &= ((__double2hiint(x[k]) >> 20) & 0x7ff) != 0x7ff;
+      asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(f[k]) : "d"(x[k]));
+    }
+  }
+  return finite;
+}
+// Requests the lines of [p, p + bytes) into the L2 (one block's share).
+__device__ __forceinline__ void prefetch_l2(const void *p, int bytes, int tid, int nth) {
+  const char *c = static_cast<const char *>(p);
+  for (int o = tid * 128; o < bytes; o += nth * 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(c + o));
+}
 // Finite test on the exponent bits of an FP64 value (integer pipe: FP64
 // compares run at the FP64 rate, which is low on this part).
 __device__ __forceinline__ bool finite64(double x) {

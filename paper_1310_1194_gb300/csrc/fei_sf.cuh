@@ -381,6 +381,16 @@ __global__ void __launch_bounds__(SfCfg<T, P>::NTH, SfCfg<T, P>::MINB) sf_forwar
   for (int64_t base = (int64_t)blockIdx.x * E; base < items; base += step, cur ^= 1) {
     const int nel = items - base < E ? (int)(items - base) : E;
     SfElem<T, P> *EL = ELS[cur];
+    // the next batch's per-point records on their way to the L2
+    if (!per_elem)
+      for (int sl = 0; sl < E && base + step + sl < items; ++sl) {
+        const int64_t it = base + step + sl, e = a.list ? (int64_t)a.list[it] : it;
+        const int64_t r = a.q_off ? a.q_off[e] : e * (int64_t)NQ;
+        prefetch_l2(a.K + 9 * r, 72 * NQ, tid, NTH);
+        prefetch_l2(a.b + 3 * r, 24 * NQ, tid, NTH);
+        prefetch_l2(a.c + r, 8 * NQ, tid, NTH);
+        prefetch_l2(a.f + r, 8 * NQ, tid, NTH);
+      }
     // ---- 2: point operators
     for (int o = tid; o < nel * NQ; o += NTH) {
       // points in the order (iv, iz, iu) of the operators' layout
@@ -393,23 +403,22 @@ __global__ void __launch_bounds__(SfCfg<T, P>::NTH, SfCfg<T, P>::MINB) sf_forwar
         const int64_t e = a.list ? (int64_t)a.list[base + sl] : base + sl;
         const int64_t r = (a.q_off ? a.q_off[e] : e * (int64_t)NQ) + q;
         double cq[14];
-        bool fin = true;
 #pragma unroll
         for (int k = 0; k < 9; ++k) cq[k] = a.K[9 * r + k];
 #pragma unroll
         for (int k = 0; k < 3; ++k) cq[9 + k] = a.b[3 * r + k];
         cq[12] = a.c[r];
         cq[13] = a.f[r];
+        T cv[14];
+        bool fin = true;
+        if constexpr (F32) {
+          fin = coef_to_f32<14>(cq, cv);
+        } else {
 #pragma unroll
-        for (int k = 0; k < 14; ++k) fin &= finite64(cq[k]);
+          for (int k = 0; k < 14; ++k) fin &= finite64(cv[k] = cq[k]);
+        }
         if (!fin) pst = FEI_ERR_NONFINITE;
         else if (UP && !coef_symmetric(cq, cq + 9)) pst = FEI_ERR_INVALID_ARG;
-        T cv[14];
-#pragma unroll
-        for (int k = 0; k < 14; ++k) {
-          if constexpr (F32) cv[k] = f64_to_f32_bits(cq[k]);
-          else cv[k] = cq[k];
-        }
 #pragma unroll
         for (int k = 0; k < 9; ++k) K[k] = cv[k];
 #pragma unroll
