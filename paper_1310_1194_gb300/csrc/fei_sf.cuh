@@ -49,24 +49,25 @@ namespace fei {
 // Elements per block (E), rows per thread (R), blocks per SM the register
 // budget is set for (MINB).  E > 1 where one element's columns and row blocks
 // do not fill warps.  Larger R reads X less often; the choices are the fastest
-// measured (GB300, FP32, against the kernel with 21 term pairs, Y in shared
-// memory and one barrier pair per term pair that this one replaced):
-//   p = 2, 200 000 prisms: 0.61 ms (dense, one warp per element: 2.51)
-//   p = 3,  60 000: 0.35 ms (1.67); R = 2: 0.41
-//   p = 4, 100 000: 1.58 ms (5.41); R = 5: 1.81, E = 4: 1.79
-//   p = 5,  20 000: 0.75 ms (1.81); R = 4, MINB = 5: 0.81
-//   p = 6,  16 384: 1.44 ms (3.8); MINB = 3 (spills): 1.70
-//   p = 7,  16 384: 2.26 ms (6.25); R = 4: 2.42, R = 5: 2.91
-// What bounds it (ncu, p = 7): issue (64 % of slots: FMA pipe 41 %, ALU 20 %),
-// with barrier and shared-memory latency as the largest stalls; DRAM writes
-// are the outputs.  FP64: the FP64 pipe (p = 4, 4096 prisms: 1.26 ms; the
+// measured (GB300, FP32; in brackets the kernels that this one replaced: the
+// dense one at p = 2, the one with 21 term pairs above):
+//   p = 2, 200 000 prisms: 0.49 ms (2.51); MINB = 8: 0.54
+//   p = 3,  60 000: 0.31 ms (1.67); R = 2: 0.36
+//   p = 4, 100 000: 1.34 ms (5.41); R = 5: 1.68, MINB = 5: 1.48
+//   p = 5,  20 000: 0.68 ms (1.81); R = 2: 0.71, MINB = 6: 0.71
+//   p = 6,  16 384: 1.28 ms (3.8); R = 3: 1.41, MINB = 3: 1.9
+//   p = 7,  16 384: 2.12 ms (6.25); R = 2: 2.26, R = 4: 2.15
+// What bounds it (ncu): issue (p = 4: 71 % of slots, 11.8 k warp instructions
+// an element; p = 7: 56 %, 91 k), with barriers and shared-memory latency as
+// the largest stalls; without its stores it takes the same time, DRAM writes
+// are the outputs.  FP64: the FP64 pipe (p = 4, 4096 prisms: 1.25 ms; the
 // dense kernel 23.2 ms).
 template <typename T, int P>
 struct SfShape;
 template <> struct SfShape<float, 2> { static constexpr int E = 4, R = 3, MINB = 6; };
 template <> struct SfShape<float, 3> { static constexpr int E = 3, R = 4, MINB = 6; };
 template <> struct SfShape<float, 4> { static constexpr int E = 2, R = 3, MINB = 4; };
-template <> struct SfShape<float, 5> { static constexpr int E = 1, R = 3, MINB = 6; };
+template <> struct SfShape<float, 5> { static constexpr int E = 1, R = 3, MINB = 5; };
 template <> struct SfShape<float, 6> { static constexpr int E = 1, R = 4, MINB = 2; };
 template <> struct SfShape<float, 7> { static constexpr int E = 1, R = 3, MINB = 2; };
 template <> struct SfShape<double, 2> { static constexpr int E = 4, R = 3, MINB = 2; };
@@ -82,6 +83,9 @@ struct SfCfg {
   static constexpr int M = P + 1, NT = M * (M + 1) / 2, NSH = nsh_of(P), NQ = nq_of(P), NT2 = M * M;
   static constexpr int E = SfShape<T, P>::E, R = SfShape<T, P>::R, MINB = SfShape<T, P>::MINB;
   static constexpr int NE = (M + 1) / 2, NO = M / 2;  // even and odd l (and half nodes of u)
+  // packed FP32 multiply-adds in the v sums; not where odd counts of l would
+  // leave halves of the packs unused and cost registers (M = 5, 6)
+  static constexpr bool PACKED = F32 && M != 5 && M != 6;
   static constexpr int NG = (M + 1) / 2;              // row groups
   static constexpr int nblk(int g) {                  // row blocks of group g
     const int c0 = M - g, c1 = g + 1;
@@ -94,10 +98,11 @@ struct SfCfg {
   }();
   static constexpr int WPC = (E * NBLK * NT + 31) / 32;  // warps per entry class
   static constexpr int NW = 2 * WPC, NTH = 32 * NW;
-  static constexpr int XR = NE > 2 ? 8 : 4; // an l row: even l, odd l (each padded)
-  // stride of an (m, m') chunk of X: an odd multiple of 4 values, so that
-  // the chunks of consecutive m' start in different banks
-  static constexpr int XS = M == 3 ? 20 : M * XR + 4;
+  // an l row of X: even l, then odd l from XO (padded for vector loads)
+  static constexpr int XR = M == 5 ? 6 : NE > 2 ? 8 : 4, XO = M == 5 ? 4 : XR / 2;
+  // stride of an (m, m') chunk of X: an odd multiple of the vector loads'
+  // size, so that the chunks of consecutive m' start in different banks
+  static constexpr int XS = M == 3 ? 20 : M == 5 ? 34 : M * XR + 4;
   static constexpr int XC = 2 * M * XS;     // one combination of a group
   // shared memory, in values of T
   static constexpr int O_D = SfTab<P>::SIZE;             // [E] operators (OpPos)
@@ -107,8 +112,16 @@ struct SfCfg {
   static constexpr int O_F = O_X + E * XE;               // [E][NQ] load weights
   static constexpr int O_F1 = O_F + (E * NQ + 3) / 4 * 4;
   static constexpr int O_F2 = O_F1 + (E * NQ + 3) / 4 * 4;
-  static constexpr int VALUES = O_F2 + (E * M * NT + 3) / 4 * 4;
-  static constexpr int DYN_SMEM = VALUES * (int)sizeof(T);
+  // v factors as packs: columns [M iv][NT t], then rows [M iv][NT r]
+  static constexpr int O_FAC = O_F2 + (E * M * NT + 3) / 4 * 4;
+  static constexpr int VALUES = O_FAC + (PACKED ? 8 : 4) * M * NT;
+  // lookup tables: per lane of the u sums its operators' and X's offsets,
+  // per column of the zeta transform its offset
+  static constexpr int PER = E * NT2, W0 = (PER + 31) / 32, W1 = W0 + (2 * PER + 31) / 32,
+                       W2 = W1 + (2 * PER + 31) / 32, W3 = W2 + (4 * PER + 31) / 32;
+  static constexpr int B_U = VALUES * (int)sizeof(T), B_Z = B_U + 4 * 32 * W3;
+  static constexpr int DYN_SMEM = B_Z + (2 * E * kOps * NT2 + 15) / 16 * 16;
+  static_assert(E * DE < 65536 && E * XE < 65535, "16-bit offsets");
   static_assert(E <= NW, "one warp per element in the setup");
 };
 
@@ -177,89 +190,154 @@ __device__ __forceinline__ void u_sum(const T *D, int sw, const T *tab, int g, T
   }
 }
 
+// Packs of values for the v sums.  FP32: pairs with packed multiply-adds (half
+// the issue slots), the v factors stored twice ({B, B, 2B', 2B'}) so that they
+// need no move into a pair.
+template <typename T, bool PACKED>
+struct Pack;
+template <>
+struct Pack<float, true> {
+  using type = float2;
+  using factors = float4;
+  static constexpr int W = 2;
+  static __device__ __forceinline__ float2 zero() { return make_float2(0.f, 0.f); }
+  static __device__ __forceinline__ float2 first(float4 f) { return make_float2(f.x, f.y); }
+  static __device__ __forceinline__ float2 second(float4 f) { return make_float2(f.z, f.w); }
+  static __device__ __forceinline__ float2 mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+  static __device__ __forceinline__ float2 fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+  static __device__ __forceinline__ float get(float2 v, int i) { return i ? v.y : v.x; }
+  template <int N, bool A16>
+  static __device__ __forceinline__ void load(const float *s, float2 *v) {
+    if constexpr (N == 2 && A16) {
+      const float4 f = *reinterpret_cast<const float4 *>(s);
+      v[0] = make_float2(f.x, f.y), v[1] = make_float2(f.z, f.w);
+    } else {
+#pragma unroll
+      for (int i = 0; i < N; ++i) v[i] = reinterpret_cast<const float2 *>(s)[i];
+    }
+  }
+  static __device__ __forceinline__ void put(float *f, int i, float b, float d) {
+    reinterpret_cast<float4 *>(f)[i] = make_float4(b, b, d, d);
+  }
+};
+template <typename T>
+struct Pack<T, false> {
+  using type = T;
+  using factors = typename Vec2<T>::type;
+  static constexpr int W = 1;
+  static __device__ __forceinline__ T zero() { return T(0); }
+  static __device__ __forceinline__ T first(factors f) { return f.x; }
+  static __device__ __forceinline__ T second(factors f) { return f.y; }
+  static __device__ __forceinline__ T mul(T a, T b) { return a * b; }
+  static __device__ __forceinline__ T fma(T a, T b, T c) { return a * b + c; }
+  static __device__ __forceinline__ T get(T v, int) { return v; }
+  template <int N, bool A16>
+  static __device__ __forceinline__ void load(const T *s, T *v) {
+    if constexpr (A16 || N <= 2) {
+      load_vec<N>(s, v);
+    } else {
+      load_vec<2>(s, v);
+      v[2] = s[2];
+    }
+  }
+  static __device__ __forceinline__ void put(T *f, int i, T b, T d) {
+    factors v;
+    v.x = b, v.y = d;
+    reinterpret_cast<factors *>(f)[i] = v;
+  }
+};
+
 // Stage 5 for one entry class CL (parity of k + k'): nr rows from n0 of
 // (m, ml) and column t2 = (m2, ...), results stored at o (row t of the first
 // row, column t2), or zeros for a flagged element.
 template <typename T, int P, int CL, bool UP>
-__device__ __forceinline__ void v_zeta_sums(const T *X, const T *tab, int ml, int m, int n0, int nr, int t2, int m2,
+__device__ __forceinline__ void v_zeta_sums(const T *X, const T *fac, int ml, int m, int n0, int nr, int t2, int m2,
                                             T *A, bool flagged) {
   using C = SfCfg<T, P>;
   constexpr int M = C::M, NT = C::NT, NSH = C::NSH, R = C::R, XR = C::XR, XS = C::XS, XC = C::XC;
   // values of l that meet LL and L'L' (same parity as the class) and LL', L'L
   constexpr int NA = CL ? C::NO : C::NE, NB = CL ? C::NE : C::NO;
-  constexpr int OA = CL ? XR / 2 : 0, OB = CL ? 0 : XR / 2;
-  using V2 = typename Vec2<T>::type;
+  constexpr int OA = CL ? C::XO : 0, OB = CL ? 0 : C::XO;
   auto row_of = [&](int r) { return tri_index(m, n0 + r); };
-  auto store = [&](int k, int k2, int t, T v) {
+  // entry (k, k') of row t; o: A_e[t][t2] (full layout)
+  auto store = [&](T *o, int k, int k2, int t, T v) {
     if constexpr (UP) {
       const int row = k * NT + t, col = k2 * NT + t2;
       if (col >= row) A[a_pos(row, col, NSH, true)] = v;
     } else {
-      A[(k * NT + t) * NSH + k2 * NT + t2] = v;
+      o[k * NT * NSH + k2 * NT] = v;
     }
   };
   if (flagged) {
     for (int r = 0; r < nr; ++r)
       for (int k = 0; k < M; ++k)
-        for (int k2 = (k + CL) & 1; k2 < M; k2 += 2) store(k, k2, row_of(r), T(0));
+        for (int k2 = (k + CL) & 1; k2 < M; k2 += 2) store(A + (row_of(r) * NSH + t2), k, k2, row_of(r), T(0));
     return;
   }
-  T a00[R][NA], a11[R][NA], a01[R][NB], a10[R][NB];
+  // PA, PB: the values of l as packs of W (FP32: pairs, one packed
+  // multiply-add each; an odd count leaves the last half unused)
+  using Pk = Pack<T, C::PACKED>;
+  constexpr bool A16 = XR % 4 == 0, ROLL = P >= 4;
+  using V = typename Pk::type;
+  constexpr int W = Pk::W, PA = (NA + W - 1) / W, PB = (NB + W - 1) / W;
+  V a00[R][PA], a11[R][PA], a01[R][PB], a10[R][PB];
 #pragma unroll
   for (int r = 0; r < R; ++r) {
 #pragma unroll
-    for (int i = 0; i < NA; ++i) a00[r][i] = a11[r][i] = T(0);
+    for (int i = 0; i < PA; ++i) a00[r][i] = a11[r][i] = Pk::zero();
 #pragma unroll
-    for (int i = 0; i < NB; ++i) a01[r][i] = a10[r][i] = T(0);
+    for (int i = 0; i < PB; ++i) a01[r][i] = a10[r][i] = Pk::zero();
   }
   const T *x0 = X + (ml * M + m2) * XS;
-  const V2 *vc = reinterpret_cast<const V2 *>(tab + SfTab<P>::O_VC) + t2;
-  const V2 *vr = reinterpret_cast<const V2 *>(tab + SfTab<P>::O_VR) + row_start(M, m) + n0;
+  const typename Pk::factors *vc = reinterpret_cast<const typename Pk::factors *>(fac) + t2;
+  const typename Pk::factors *vr = reinterpret_cast<const typename Pk::factors *>(fac) + M * NT + row_start(M, m) + n0;
 #pragma unroll 1
   for (int iv = 0; iv < M; ++iv) {
-    const V2 vb = vc[iv * NT];
+    const typename Pk::factors fb = vc[iv * NT];
+    const V b0 = Pk::first(fb), b1 = Pk::second(fb);
     const T *xa = x0 + iv * XR + OA, *xb = x0 + iv * XR + OB;
-    T za[NA], zb[NA], zc[NA], zd[NB], ze[NB], zf[NB];
+    V za[PA], zb[PA], zc[PA], zd[PB], ze[PB], zf[PB];
     {
-      T p[NA], q[NA];
-      load_vec<NA>(xa, p);
-      load_vec<NA>(xa + XC, q);
+      V p[PA], q[PA];
+      Pk::template load<PA, A16>(xa, p);
+      Pk::template load<PA, A16>(xa + XC, q);
 #pragma unroll
-      for (int i = 0; i < NA; ++i) za[i] = vb.x * p[i] + vb.y * q[i];
-      load_vec<NA>(xa + 2 * XC, p);
-      load_vec<NA>(xa + 3 * XC, q);
+      for (int i = 0; i < PA; ++i) za[i] = Pk::fma(b1, q[i], Pk::mul(b0, p[i]));
+      Pk::template load<PA, A16>(xa + 2 * XC, p);
+      Pk::template load<PA, A16>(xa + 3 * XC, q);
 #pragma unroll
-      for (int i = 0; i < NA; ++i) zb[i] = vb.x * p[i] + vb.y * q[i];
-      load_vec<NA>(xa + 8 * XC, p);
+      for (int i = 0; i < PA; ++i) zb[i] = Pk::fma(b1, q[i], Pk::mul(b0, p[i]));
+      Pk::template load<PA, A16>(xa + 8 * XC, p);
 #pragma unroll
-      for (int i = 0; i < NA; ++i) zc[i] = vb.x * p[i];
+      for (int i = 0; i < PA; ++i) zc[i] = Pk::mul(b0, p[i]);
     }
     {
-      T p[NB], q[NB];
-      load_vec<NB>(xb + 4 * XC, p);
-      load_vec<NB>(xb + 5 * XC, q);
+      V p[PB], q[PB];
+      Pk::template load<PB, A16>(xb + 4 * XC, p);
+      Pk::template load<PB, A16>(xb + 5 * XC, q);
 #pragma unroll
-      for (int i = 0; i < NB; ++i) zd[i] = vb.x * p[i], ze[i] = vb.x * q[i];
-      load_vec<NB>(xb + 6 * XC, p);
-      load_vec<NB>(xb + 7 * XC, q);
+      for (int i = 0; i < PB; ++i) zd[i] = Pk::mul(b0, p[i]), ze[i] = Pk::mul(b0, q[i]);
+      Pk::template load<PB, A16>(xb + 6 * XC, p);
+      Pk::template load<PB, A16>(xb + 7 * XC, q);
 #pragma unroll
-      for (int i = 0; i < NB; ++i) zf[i] = vb.x * p[i] + vb.y * q[i];
+      for (int i = 0; i < PB; ++i) zf[i] = Pk::fma(b1, q[i], Pk::mul(b0, p[i]));
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       if (r < nr) {
-        const V2 va = vr[iv * NT + r];
+        const typename Pk::factors fa = vr[iv * NT + r];
+        const V c0 = Pk::first(fa), c1 = Pk::second(fa);
 #pragma unroll
-        for (int i = 0; i < NA; ++i) {
-          a00[r][i] += va.x * za[i];
-          a00[r][i] += va.y * zb[i];
-          a11[r][i] += va.x * zc[i];
+        for (int i = 0; i < PA; ++i) {
+          a00[r][i] = Pk::fma(c0, za[i], a00[r][i]);
+          a00[r][i] = Pk::fma(c1, zb[i], a00[r][i]);
+          a11[r][i] = Pk::fma(c0, zc[i], a11[r][i]);
         }
 #pragma unroll
-        for (int i = 0; i < NB; ++i) {
-          a01[r][i] += va.x * zd[i];
-          a01[r][i] += va.y * ze[i];
-          a10[r][i] += va.x * zf[i];
+        for (int i = 0; i < PB; ++i) {
+          a01[r][i] = Pk::fma(c0, zd[i], a01[r][i]);
+          a01[r][i] = Pk::fma(c1, ze[i], a01[r][i]);
+          a10[r][i] = Pk::fma(c0, zf[i], a10[r][i]);
         }
       }
     }
@@ -268,10 +346,16 @@ __device__ __forceinline__ void v_zeta_sums(const T *X, const T *tab, int ml, in
   // contribute alike to (k, k') and (k', k), and LL' to one what L'L does to
   // the other: with the sum and the difference of Y01 and Y10 an entry pair
   // takes half the terms of its two entries.
-  auto zeta_row = [&](int t, const T *r00, const T *r11, const T *r01, const T *r10) {
-    T ps[NB], pd[NB];
+  auto zeta_row = [&](int t, const V *v00, const V *v11, const V *v01, const V *v10) {
+    T *o = A + (t * NSH + t2);
+    T r00[NA], r11[NA], ps[NB], pd[NB];
 #pragma unroll
-    for (int i = 0; i < NB; ++i) ps[i] = r01[i] + r10[i], pd[i] = r01[i] - r10[i];
+    for (int i = 0; i < NA; ++i) r00[i] = Pk::get(v00[i / W], i % W), r11[i] = Pk::get(v11[i / W], i % W);
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      const T y01 = Pk::get(v01[i / W], i % W), y10 = Pk::get(v10[i / W], i % W);
+      ps[i] = y01 + y10, pd[i] = y01 - y10;
+    }
     static_for<M>([&](auto k) {
       static_for<M - k.value>([&](auto dk) {
         constexpr int ka = k.value, kb = ka + dk.value;
@@ -291,18 +375,34 @@ __device__ __forceinline__ void v_zeta_sums(const T *X, const T *tab, int ml, in
             if constexpr (ka != kb && (hd > 1e-11 || hd < -1e-11)) d += T(hd) * pd[i.value];
           });
           if constexpr (ka == kb) {
-            store(ka, ka, t, s);
+            store(o, ka, ka, t, s);
           } else {
-            store(ka, kb, t, s + d);
-            store(kb, ka, t, s - d);
+            store(o, ka, kb, t, s + d);
+            store(o, kb, ka, t, s - d);
           }
         }
       });
     });
   };
+  if constexpr (ROLL) {
+    // the next row's values move down: the code of the entries exists once
+    // (unrolled rows miss the instruction cache: p = 4 1.38, p = 7 2.21 ms)
+#pragma unroll 1
+    for (int r = 0; r < nr; ++r) {
+      zeta_row(row_of(r), a00[0], a11[0], a01[0], a10[0]);
 #pragma unroll
-  for (int r = 0; r < R; ++r)
-    if (r < nr) zeta_row(row_of(r), a00[r], a11[r], a01[r], a10[r]);
+      for (int j = 0; j + 1 < R; ++j) {
+#pragma unroll
+        for (int i = 0; i < PA; ++i) a00[j][i] = a00[j + 1][i], a11[j][i] = a11[j + 1][i];
+#pragma unroll
+        for (int i = 0; i < PB; ++i) a01[j][i] = a01[j + 1][i], a10[j][i] = a10[j + 1][i];
+      }
+    }
+  } else {
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      if (r < nr) zeta_row(row_of(r), a00[r], a11[r], a01[r], a10[r]);
+  }
 }
 
 template <typename T, int P, bool UP>
@@ -324,6 +424,32 @@ __global__ void __launch_bounds__(SfCfg<T, P>::NTH, SfCfg<T, P>::MINB) sf_forwar
     for (int t = tid; t < NT2; t += NTH)
       nodes.tx[t][0] = a.tnode[4 * t], nodes.tx[t][1] = a.tnode[4 * t + 1], nodes.tw[t] = a.tnode[4 * t + 2];
     for (int z = tid; z < M; z += NTH) nodes.zz[z] = a.znode[2 * z], nodes.zw[z] = a.znode[2 * z + 1];
+  }
+  T *fac = sm + C::O_FAC;
+  for (int i = tid; i < 2 * M * NT; i += NTH) {
+    const T *v = gtab + SfTab<P>::O_VC + 2 * i;  // VC, then VR (M NT pairs each)
+    static_assert(SfTab<P>::O_VR == SfTab<P>::O_VC + (2 * M * NT + 3) / 4 * 4, "VR after VC");
+    const T *w = i < M * NT ? v : gtab + SfTab<P>::O_VR + 2 * (i - M * NT);
+    Pack<T, C::PACKED>::put(fac, i, w[0], w[1]);
+  }
+  uint32_t *tabu = reinterpret_cast<uint32_t *>(smraw + C::B_U);
+  uint16_t *tabz = reinterpret_cast<uint16_t *>(smraw + C::B_Z);
+  // u sums: combinations with the same kinds of pairs share warps: 0 | 1 4 |
+  // 2 6 | 3 5 7 8 (most pairs first); entry: the offset of the first pair's
+  // u row (its low bits l & 4 where halves are swapped) and of X
+  for (int i = tid; i < 32 * C::W3; i += NTH) {
+    const int wt = i >> 5, kind = (wt >= C::W0) + (wt >= C::W1) + (wt >= C::W2);
+    const int li = i - 32 * (kind == 0 ? 0 : kind == 1 ? C::W0 : kind == 2 ? C::W1 : C::W2), j = li / C::PER,
+              i0 = li - j * C::PER, sl = i0 / NT2, t = i0 - sl * NT2, iv = t / M, l = t - iv * M;
+    const int op = kind == 0 ? 0 : kind == 1 ? 2 + j : kind == 2 ? 7 + 3 * j : (0xCB98 >> (4 * j)) & 15;
+    const int ci = kind == 0 ? 0 : kind == 1 ? 1 + 3 * j : kind == 2 ? 2 + 4 * j : (0x8753 >> (4 * j)) & 15;
+    const uint32_t dof = sl * C::DE + OpPos<T, M>::row(op, iv, l) + (OpPos<T, M>::SWZ ? l & 4 : 0);
+    const uint32_t xof = sl * C::XE + ci * XC + iv * XR + (l & 1) * C::XO + (l >> 1);
+    tabu[i] = j < (kind == 0 ? 1 : kind == 3 ? 4 : 2) ? dof | xof << 16 : 0xffffffffu;
+  }
+  for (int i = tid; i < E * kOps * NT2; i += NTH) {
+    const int sl = i / (kOps * NT2), i0 = i - sl * (kOps * NT2), k = i0 / NT2, t = i0 - k * NT2, iv = t / M;
+    tabz[i] = (uint16_t)(sl * C::DE + OpPos<T, M>::row(k, iv, 0) + t - iv * M);
   }
   const T *gv = sm + SfTab<P>::O_GV, *su = sm + SfTab<P>::O_SU, *mtf = sm + SfTab<P>::O_MT;
   const int64_t items = a.count ? (int64_t)(*a.count) : a.n_work;
@@ -463,12 +589,12 @@ __global__ void __launch_bounds__(SfCfg<T, P>::NTH, SfCfg<T, P>::MINB) sf_forwar
     __syncthreads();
     // ---- 3: zeta transform, d^_l = sum_i L_l(z_i) d_i, even and odd l
     for (int o = tid; o < nel * kOps * NT2; o += NTH) {
-      const int sl = o / (kOps * NT2), i0 = o - sl * (kOps * NT2), k = i0 / NT2, t = i0 - k * NT2, iv = t / M,
-                iu = t - iv * M;
-      T *col = D + sl * C::DE;
+      // the column (op, iv, iu) at stride M in l (halves swapped by l & 4)
+      const int c0 = tabz[o];
+      auto at = [&](int l) { return (OpPos<T, M>::SWZ ? c0 ^ (l & 4) : c0) + l * M; };
       T d[M];
 #pragma unroll
-      for (int i = 0; i < M; ++i) d[i] = col[OpPos<T, M>::at(k, iv, i, iu)];
+      for (int i = 0; i < M; ++i) d[i] = D[at(i)];
       T ev[C::NE], od[C::NE];
 #pragma unroll
       for (int i = 0; i < C::NE; ++i) {
@@ -482,7 +608,7 @@ __global__ void __launch_bounds__(SfCfg<T, P>::NTH, SfCfg<T, P>::MINB) sf_forwar
           constexpr double c = Leg<M>::tab.L[l.value][i.value];
           if constexpr (c != 0.0) s += T(c) * (l.value % 2 ? od[i.value] : ev[i.value]);
         });
-        col[OpPos<T, M>::at(k, iv, l.value, iu)] = s;
+        D[at(l.value)] = s;
       });
     }
     __syncthreads();
@@ -492,39 +618,29 @@ __global__ void __launch_bounds__(SfCfg<T, P>::NTH, SfCfg<T, P>::MINB) sf_forwar
       const bool single = 2 * g == M - 1;
       // ---- 4: u sums, lanes over (combination, iv, l)
       {
-        // combinations with the same kinds of pairs share warps: 0 | 1 4 |
-        // 2 6 | 3 5 7 8 (most pairs first)
-        const int per = nel * NT2;
-        const int w0 = (per + 31) / 32, w1 = w0 + (2 * per + 31) / 32, w2 = w1 + (2 * per + 31) / 32,
-                  w3 = w2 + (4 * per + 31) / 32;
-        for (int wt = warp; wt < w3; wt += NW) {
-          const int kind = (wt >= w0) + (wt >= w1) + (wt >= w2);
-          const int li = (wt - (kind == 0 ? 0 : kind == 1 ? w0 : kind == 2 ? w1 : w2)) * 32 + lane, j = li / per,
-                    i0 = li - j * per, sl = i0 / NT2, t = i0 - sl * NT2, iv = t / M, l = t - iv * M;
-          if (j >= (kind == 0 ? 1 : kind == 3 ? 4 : 2)) continue;
+        for (int wt = warp; wt < C::W3; wt += NW) {
+          const uint32_t ent = tabu[32 * wt + lane];
+          const int dof = ent & 0xffffu, xof = ent >> 16;
+          if (ent == 0xffffffffu || dof >= nel * C::DE) continue;
           T x[2][M];
 #pragma unroll
           for (int i = 0; i < M; ++i) x[0][i] = x[1][i] = T(0);
-          const T *Dd = D + sl * C::DE + OpPos<T, M>::row(0, iv, l);
           constexpr int OP = OpPos<T, M>::OP;
-          const int sw = l & 4;
-          int ci = 0;
-          if (kind == 0) {
+          const int sw = OpPos<T, M>::SWZ ? dof & 4 : 0;
+          const T *Dd = D + dof - sw;
+          if (wt < C::W0) {
             u_sum<T, P, 0, 0>(Dd, sw, sm, g, x);
             u_sum<T, P, 0, 1>(Dd + OP, sw, sm, g, x);
             u_sum<T, P, 1, 1>(Dd + 4 * OP, sw, sm, g, x);
-          } else if (kind == 1) {
-            ci = 1 + 3 * j;
-            u_sum<T, P, 0, 0>(Dd + (2 + j) * OP, sw, sm, g, x);
-            u_sum<T, P, 1, 0>(Dd + (5 + j) * OP, sw, sm, g, x);
-          } else if (kind == 2) {
-            ci = 2 + 4 * j;
-            u_sum<T, P, 0, 1>(Dd + (7 + 3 * j) * OP, sw, sm, g, x);
+          } else if (wt < C::W1) {
+            u_sum<T, P, 0, 0>(Dd, sw, sm, g, x);
+            u_sum<T, P, 1, 0>(Dd + 3 * OP, sw, sm, g, x);
+          } else if (wt < C::W2) {
+            u_sum<T, P, 0, 1>(Dd, sw, sm, g, x);
           } else {
-            ci = (0x8753 >> (4 * j)) & 15;
-            u_sum<T, P, 0, 0>(Dd + ((0xCB98 >> (4 * j)) & 15) * OP, sw, sm, g, x);
+            u_sum<T, P, 0, 0>(Dd, sw, sm, g, x);
           }
-          T *dst = X + sl * C::XE + ci * XC + iv * XR + (l & 1) * (XR / 2) + (l >> 1);
+          T *dst = X + xof;
 #pragma unroll
           for (int m2 = 0; m2 < M; ++m2) dst[m2 * XS] = x[0][m2];
           if (!single) {
@@ -566,8 +682,8 @@ __global__ void __launch_bounds__(SfCfg<T, P>::NTH, SfCfg<T, P>::MINB) sf_forwar
           const T *Xs = X + sl * C::XE;
           const int m2 = (int)mtf[t2];
           const bool flagged = EL[sl].status != 0;
-          if (cl == 0) v_zeta_sums<T, P, 0, UP>(Xs, sm, ml, m, n0, nr, t2, m2, A, flagged);
-          else v_zeta_sums<T, P, 1, UP>(Xs, sm, ml, m, n0, nr, t2, m2, A, flagged);
+          if (cl == 0) v_zeta_sums<T, P, 0, UP>(Xs, fac, ml, m, n0, nr, t2, m2, A, flagged);
+          else v_zeta_sums<T, P, 1, UP>(Xs, fac, ml, m, n0, nr, t2, m2, A, flagged);
         }
         if (g == 0) {
           for (int o = tid; o < nel * M * NT; o += NTH) {
