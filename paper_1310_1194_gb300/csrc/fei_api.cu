@@ -63,21 +63,12 @@ fei_status workspace_for(int dev, int64_t n, Workspace **out) {
   return FEI_OK;
 }
 
-// One atomic per element into the bucket of its degree; elements whose
-// degree has no reference (avail bit clear) or lies outside 1..7 get
-// FEI_ERR_INVALID_DEGREE in their status and no bucket.
+// Elements into the buckets of their degrees; elements whose degree has no
+// reference (avail bit clear) or lies outside 1..7 get FEI_ERR_INVALID_DEGREE
+// in their status (if given) and no bucket.
 __global__ void bucket_kernel(const int32_t *degree, int64_t n, unsigned avail, int32_t *counts,
                               int32_t *lists, int64_t cap, int32_t *status) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int p = degree[e];
-    if (p >= 1 && p <= kPMax && ((avail >> p) & 1u)) {
-      const int pos = atomicAdd(&counts[p], 1);
-      lists[(int64_t)(p - 1) * cap + pos] = (int32_t)e;
-    } else if (status) {
-      status[e] = FEI_ERR_INVALID_DEGREE;
-    }
-  }
+  bucket_elements(degree, n, avail, counts, lists, cap, status);
 }
 
 // Single-block exclusive scan of N_sh^2, N_sh and N_q over the degrees.

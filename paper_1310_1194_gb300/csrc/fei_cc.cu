@@ -11,6 +11,8 @@
 // vertical-node sums of det J in FP64, w det J at every point in double-FP32
 // rounded once; the adjugate rows, the point operator and the contraction in
 // FP32.
+#include <type_traits>
+
 #include "fei_geom.cuh"
 #include "fei_internal.cuh"
 
@@ -229,22 +231,24 @@ __global__ void __launch_bounds__(SmallCfg::WPB * 32) cc_small_kernel(FwdArgs a)
 // ---------------------------------------------------------------------------
 // p = 1, FP32 path: one thread per element.  A p = 1 element is small (6
 // shape functions, 8 points, 36 entries), so a thread keeps A_e and b_e in
-// registers and runs the points in turn.  With one element per lane, every
-// FP64 instruction of the setup (element vectors, the vertical-node sums
-// of det J) serves 32 elements: this part's FP64 rate is what binds p = 1,
-// and a warp shared by four elements ran most of that work on a few lanes.
+// registers and runs the points in turn.  Records and results pass through
+// shared memory, so that consecutive threads touch consecutive addresses (a
+// thread's own record or matrix is a line of its own in every load and
+// store).  1 000 000 prisms (GB300): 0.275 ms, 1.56 TB/s of inputs and
+// outputs; with FP64 node sums and per-thread loads and stores 0.467 ms.  It
+// is bound by issue (51 % of slots with the 12 warps an SM that the
+// registers allow); more blocks per SM spill (4: 0.30, 5: 0.38 ms).
 // ---------------------------------------------------------------------------
 constexpr int kP1Threads = 128;
 
 // The two p = 1 kernels below (one thread per element for large batches,
 // eight lanes per element for small ones) give the same bits: their
-// FP64 node sums and their sums over points run in one fixed order of
+// node sums and their sums over points run in one fixed order of
 // rounded operations (the host-memory entry cuts a batch into chunks of
 // any size and must equal the device entry bit for bit).
 //
-// w_z (n3.C, n3.D1, n3.D2) of a vertical node as FP32 pairs, from the
-// columns' components c1[k], c2[k] and C, D1, D2 (FP64): n3_k and its
-// products p_k rounded one by one, value v summed as (p_v + p_v+1) + p_v+2.
+// FP64 node sums (p1_setup64): n3_k and its products p_k rounded one by one,
+// value v summed as (p_v + p_v+1) + p_v+2.
 __device__ __forceinline__ double p1_node_sum(const double *n3, const double *w, int v) {
   const double a = __dmul_rn(n3[v], w[v]), b = __dmul_rn(n3[(v + 1) % 3], w[(v + 1) % 3]);
   const double c = __dmul_rn(n3[(v + 2) % 3], w[(v + 2) % 3]);
@@ -253,32 +257,141 @@ __device__ __forceinline__ double p1_node_sum(const double *n3, const double *w,
 __device__ __forceinline__ double p1_cross_comp(double a1, double a2, double b1, double b2) {
   return __dsub_rn(__dmul_rn(a1, b2), __dmul_rn(a2, b1));  // a1 b2 - a2 b1
 }
+// The gradient components of p = 1 function i = 3 k + t that are not zero
+// everywhere, as bits (1: d/dxi1, 2: d/dxi2, 4: d/dzeta): t = (0,0), (1,0),
+// (0,1) with L_0 constant and L_1 linear in zeta.
+__host__ __device__ constexpr int p1_grad(int i) { return (i % 3 == 1 ? 3 : i % 3 == 2 ? 2 : 0) | (i >= 3 ? 4 : 0); }
 // One point's contribution to A_e (36 values, row-major) and b_e (6):
-// G_q^T Dt_q G_q and (w det J f) G_q0, every operation rounded in turn.
+// G_q^T Dt_q G_q and (w det J f) G_q0, every operation rounded in turn, the
+// zero components left out (15 of 24 values remain).
 __device__ __forceinline__ void p1_point_contrib(const float *D, const float *G, float *c) {
   constexpr int NSH = 6;
 #pragma unroll
   for (int i = 0; i < NSH; ++i) {
-    const float g0 = G[i], g1 = G[NSH + i], g2 = G[2 * NSH + i], g3 = G[3 * NSH + i];
+    const float g0 = G[i];
     const float h0 = __fmul_rn(D[0], g0);
-    const float h1 = __fmaf_rn(D[10], g3, __fmaf_rn(D[7], g2, __fmaf_rn(D[4], g1, __fmul_rn(D[1], g0))));
-    const float h2 = __fmaf_rn(D[11], g3, __fmaf_rn(D[8], g2, __fmaf_rn(D[5], g1, __fmul_rn(D[2], g0))));
-    const float h3 = __fmaf_rn(D[12], g3, __fmaf_rn(D[9], g2, __fmaf_rn(D[6], g1, __fmul_rn(D[3], g0))));
+    float h1 = __fmul_rn(D[1], g0), h2 = __fmul_rn(D[2], g0), h3 = __fmul_rn(D[3], g0);
+    if (p1_grad(i) & 1) {
+      const float g = G[NSH + i];
+      h1 = __fmaf_rn(D[4], g, h1), h2 = __fmaf_rn(D[5], g, h2), h3 = __fmaf_rn(D[6], g, h3);
+    }
+    if (p1_grad(i) & 2) {
+      const float g = G[2 * NSH + i];
+      h1 = __fmaf_rn(D[7], g, h1), h2 = __fmaf_rn(D[8], g, h2), h3 = __fmaf_rn(D[9], g, h3);
+    }
+    if (p1_grad(i) & 4) {
+      const float g = G[3 * NSH + i];
+      h1 = __fmaf_rn(D[10], g, h1), h2 = __fmaf_rn(D[11], g, h2), h3 = __fmaf_rn(D[12], g, h3);
+    }
 #pragma unroll
-    for (int j = 0; j < NSH; ++j)
-      c[i * NSH + j] = __fmaf_rn(h3, G[3 * NSH + j],
-                                 __fmaf_rn(h2, G[2 * NSH + j], __fmaf_rn(h1, G[NSH + j], __fmul_rn(h0, G[j]))));
+    for (int j = 0; j < NSH; ++j) {
+      float v = __fmul_rn(h0, G[j]);
+      if (p1_grad(j) & 1) v = __fmaf_rn(h1, G[NSH + j], v);
+      if (p1_grad(j) & 2) v = __fmaf_rn(h2, G[2 * NSH + j], v);
+      if (p1_grad(j) & 4) v = __fmaf_rn(h3, G[3 * NSH + j], v);
+      c[i * NSH + j] = v;
+    }
     c[NSH * NSH + i] = __fmul_rn(D[13], g0);
+  }
+}
+
+// Element setup.  The vertex differences are FP64 subtractions, split from
+// their bit fields into FP32 pairs; everything after them is double-FP32
+// arithmetic in operations that are rounded one by one (no contraction), so
+// that both kernels give the same bits: 21 FP64 instructions an element
+// instead of about 190 (this part's FP64 rate bound the kernel), at an error
+// of about 2^-44 before the single rounding of w det J.
+__device__ __forceinline__ float2 p1_mul(float2 a, float2 b) {
+  const float p = __fmul_rn(a.x, b.x);
+  float e = __fmaf_rn(a.x, b.x, -p);
+  e = __fmaf_rn(a.x, b.y, e);
+  e = __fmaf_rn(a.y, b.x, e);
+  return make_float2(p, e);
+}
+__device__ __forceinline__ float2 p1_add(float2 a, float2 b) {
+  const float s = __fadd_rn(a.x, b.x), bb = __fadd_rn(s, -a.x);
+  const float err = __fadd_rn(__fadd_rn(a.x, -__fadd_rn(s, -bb)), __fadd_rn(b.x, -bb));
+  return make_float2(s, __fadd_rn(__fadd_rn(err, a.y), b.y));
+}
+__device__ __forceinline__ float2 p1_norm(float2 a) {
+  const float s = __fadd_rn(a.x, a.y), bb = __fadd_rn(s, -a.x);
+  return make_float2(s, __fadd_rn(__fadd_rn(a.x, -__fadd_rn(s, -bb)), __fadd_rn(a.y, -bb)));
+}
+// half of t1 + t2
+__device__ __forceinline__ float2 p1_half_sum(float2 t1, float2 t2) {
+  const float2 v = p1_norm(p1_add(t1, t2));
+  return make_float2(__fmul_rn(0.5f, v.x), __fmul_rn(0.5f, v.y));
+}
+// Component j = 3 v + axis of the element vectors A1, B1, A2, B2, C, D1, D2 as
+// a pair (the vertices and signs of elem_vec_comp); clears *in_range where a
+// difference is outside the pairs' range.
+__device__ __forceinline__ float2 elem_vec_pair(const double *X, int j, bool *in_range) {
+  const int v = j / 3, k = j - 3 * v;
+  const int code = v == 0 ? (1 | 0 << 4 | 4 << 8 | 3 << 12 | 2 << 16)
+                   : v == 1 ? (4 | 3 << 4 | 1 << 8 | 0 << 12 | 0 << 16)
+                   : v == 2 ? (2 | 0 << 4 | 5 << 8 | 3 << 12 | 2 << 16)
+                   : v == 3 ? (5 | 3 << 4 | 2 << 8 | 0 << 12 | 0 << 16)
+                   : v == 4 ? (3 | 0 << 4 | 0 << 8 | 0 << 12 | 1 << 16)
+                   : v == 5 ? (4 | 1 << 4 | 3 << 8 | 0 << 12 | 0 << 16)
+                            : (5 | 2 << 4 | 3 << 8 | 0 << 12 | 0 << 16);
+  const double d1 = X[3 * (code & 15) + k] - X[3 * ((code >> 4) & 15) + k];
+  const double d2 = X[3 * ((code >> 8) & 15) + k] - X[3 * ((code >> 12) & 15) + k];
+  bool r1, r2;
+  const float2 t1 = split_f64_bits(d1, &r1), t2 = split_f64_bits(d2, &r2);
+  *in_range &= r1 && r2;
+  return p1_half_sum(t1, code >> 16 == 0 ? neg_ff(t2) : t2);
+}
+// component z B + A of a column
+__device__ __forceinline__ float2 p1_column(float2 z, float2 A, float2 B) { return p1_norm(p1_add(A, p1_mul(z, B))); }
+// a1 b2 - a2 b1
+__device__ __forceinline__ float2 p1_cross_pair(float2 a1, float2 a2, float2 b1, float2 b2) {
+  return p1_norm(p1_add(p1_mul(a1, b2), neg_ff(p1_mul(a2, b1))));
+}
+// (p_v + p_v+1) + p_v+2
+__device__ __forceinline__ float2 p1_sum3(float2 a, float2 b, float2 c) { return p1_norm(p1_add(p1_add(a, b), c)); }
+
+// The same setup in FP64, for an element with a vertex difference outside
+// 2^-60 <= |d| < 2^60 (other than 0): ev32 [21], then the node sums [2][3]
+// as pairs (12 values).  Not inlined: the compiler would execute its FP64
+// instructions ahead of the branch.
+__device__ __noinline__ void p1_setup64(const double *X, const double *zd, const double *zwd, float *out) {
+  double ev[21];
+  elem_vectors(X, ev);
+#pragma unroll
+  for (int k = 0; k < 21; ++k) out[k] = (float)ev[k];
+#pragma unroll
+  for (int iz = 0; iz < 2; ++iz) {
+    double c1[3], c2[3], n3[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      c1[k] = fma(zd[iz], ev[3 + k], ev[k]);
+      c2[k] = fma(zd[iz], ev[9 + k], ev[6 + k]);
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      n3[k] = p1_cross_comp(c1[(k + 1) % 3], c1[(k + 2) % 3], c2[(k + 1) % 3], c2[(k + 2) % 3]);
+#pragma unroll
+    for (int v = 0; v < 3; ++v) {
+      const float2 z = split_f64(__dmul_rn(zwd[iz], p1_node_sum(n3, ev + 12 + 3 * v, v)));
+      out[21 + 6 * iz + 2 * v] = z.x;
+      out[22 + 6 * iz + 2 * v] = z.y;
+    }
   }
 }
 
 __global__ void __launch_bounds__(kP1Threads, 3) cc_p1_kernel(FwdArgs a) {
   constexpr int NSH = 6, NQ = 8, M = 2, NT = 4;
+  constexpr int IN = 33, OUT = 43;  // odd strides: a column of the tile in distinct banks
+  // a tile's records (18 vertex coordinates, 14 coefficients), then its outputs
+  __shared__ __align__(16) double tile[kP1Threads * IN];
+  __shared__ int32_t eid[kP1Threads];
+  float *outs = reinterpret_cast<float *>(tile);
   __shared__ float Gs[4 * NQ * NSH];  // G32 [q][a][i]
   __shared__ float2 ttab[NT][3];      // w_t, w_t xi1, w_t xi2 as FP32 pairs
   __shared__ float ttabf[NT][3];      // w_t, xi1, xi2
   __shared__ float zf[M], zwf[M];
   __shared__ double zd[M], zwd[M];
+  __shared__ float2 zp[M], zwp[M];
   for (int k = threadIdx.x; k < 4 * NQ * NSH; k += blockDim.x) Gs[k] = a.G32[k];
   if (threadIdx.x < NT) {
     const int t = threadIdx.x;
@@ -295,39 +408,118 @@ __global__ void __launch_bounds__(kP1Threads, 3) cc_p1_kernel(FwdArgs a) {
     zwd[iz] = a.znode[2 * iz + 1];
     zf[iz] = (float)zd[iz];
     zwf[iz] = (float)zwd[iz];
+    zp[iz] = split_f64(zd[iz]);
+    zwp[iz] = split_f64(zwd[iz]);
   }
-  __syncthreads();
   const int64_t items = n_items(a);
-  for (int64_t item = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; item < items;
-       item += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t e = a.list ? (int64_t)a.list[item] : item;
+  const int tid = threadIdx.x;
+  const bool perq = a.coef_mode == FEI_COEF_PER_POINT;
+  const bool flat = !a.A_off && !a.b_off && !a.list && !a.upper && ((uintptr_t)a.A & 15) == 0 && ((uintptr_t)a.bv & 7) == 0;
+  for (int64_t base = blockIdx.x * (int64_t)kP1Threads; base < items; base += (int64_t)gridDim.x * kP1Threads) {
+    const int nt = items - base < kP1Threads ? (int)(items - base) : kP1Threads;
+    // the tile's records by consecutive threads (one thread per element would
+    // touch a line per lane and load)
+    if (tid < nt) eid[tid] = a.list ? a.list[base + tid] : (int32_t)(base + tid);
+    __syncthreads();
+    // (all loads of a tile in flight before the first store)
+    double in_reg[32];
+    auto gather = [&](const double *src, auto width, int at) {
+      constexpr int W = decltype(width)::value;
+#pragma unroll
+      for (int j = 0; j < W; ++j) {
+        const int i = tid + j * kP1Threads, el = i / W, k = i - el * W;
+        in_reg[at + j] = i < nt * W ? src[(int64_t)eid[el] * W + k] : 0.0;
+      }
+    };
+    auto spread = [&](auto width, int at) {
+      constexpr int W = decltype(width)::value;
+#pragma unroll
+      for (int j = 0; j < W; ++j) {
+        const int i = tid + j * kP1Threads, el = i / W, k = i - el * W;
+        tile[el * IN + at + k] = in_reg[at + j];
+      }
+    };
+    using W18 = std::integral_constant<int, 18>;
+    using W9 = std::integral_constant<int, 9>;
+    using W3 = std::integral_constant<int, 3>;
+    using W1 = std::integral_constant<int, 1>;
+    gather(a.geom, W18{}, 0);
+    if (!perq) {
+      gather(a.K, W9{}, 18);
+      gather(a.b, W3{}, 27);
+      gather(a.c, W1{}, 30);
+      gather(a.f, W1{}, 31);
+    }
+    spread(W18{}, 0);
+    if (!perq) {
+      spread(W9{}, 18);
+      spread(W3{}, 27);
+      spread(W1{}, 30);
+      spread(W1{}, 31);
+    }
+    __syncthreads();
+    // threads past the tile compute on its first record and store nothing
+    const int slot = tid < nt ? tid : 0;
+    const int64_t e = eid[slot];
+    const double *in = tile + slot * IN;
     bool ok = true, sym = true;
     float ev32[21];   // element vectors rounded once
     float2 zab[M][3];  // per vertical node w_z (n3.C, n3.D1, n3.D2), FP32 pairs
     {
-      double X[18], ev[21];
+      double X[18];
 #pragma unroll
       for (int k = 0; k < 18; ++k) {
-        X[k] = a.geom[18 * e + k];
+        X[k] = in[k];
         ok &= finite64(X[k]);
       }
-      elem_vectors(X, ev);
+      bool in_range = true;
+      float2 ev[21];
 #pragma unroll
-      for (int k = 0; k < 21; ++k) ev32[k] = (float)ev[k];
+      for (int k = 0; k < 3; ++k) {
+        auto diff = [&](int i, int j) {
+          bool r;
+          const float2 d = split_f64_bits(X[3 * i + k] - X[3 * j + k], &r);
+          in_range &= r;
+          return d;
+        };
+        const float2 e1p = diff(1, 0), e1q = diff(4, 3), e2p = diff(2, 0), e2q = diff(5, 3);
+        const float2 v0 = diff(3, 0), v1 = diff(4, 1), v2 = diff(5, 2);
+        ev[0 + k] = p1_half_sum(e1p, e1q);
+        ev[3 + k] = p1_half_sum(e1q, neg_ff(e1p));
+        ev[6 + k] = p1_half_sum(e2p, e2q);
+        ev[9 + k] = p1_half_sum(e2q, neg_ff(e2p));
+        ev[12 + k] = p1_half_sum(v0, make_float2(0.f, 0.f));
+        ev[15 + k] = p1_half_sum(v1, neg_ff(v0));
+        ev[18 + k] = p1_half_sum(v2, neg_ff(v0));
+      }
+#pragma unroll
+      for (int k = 0; k < 21; ++k) ev32[k] = ev[k].x;
 #pragma unroll
       for (int iz = 0; iz < M; ++iz) {
-        double c1[3], c2[3], n3[3];
+        float2 c1[3], c2[3], n3[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-          c1[k] = fma(zd[iz], ev[3 + k], ev[k]);
-          c2[k] = fma(zd[iz], ev[9 + k], ev[6 + k]);
+          c1[k] = p1_column(zp[iz], ev[k], ev[3 + k]);
+          c2[k] = p1_column(zp[iz], ev[6 + k], ev[9 + k]);
         }
 #pragma unroll
         for (int k = 0; k < 3; ++k)
-          n3[k] = p1_cross_comp(c1[(k + 1) % 3], c1[(k + 2) % 3], c2[(k + 1) % 3], c2[(k + 2) % 3]);
-        zab[iz][0] = split_f64(__dmul_rn(zwd[iz], p1_node_sum(n3, ev + 12, 0)));
-        zab[iz][1] = split_f64(__dmul_rn(zwd[iz], p1_node_sum(n3, ev + 15, 1)));
-        zab[iz][2] = split_f64(__dmul_rn(zwd[iz], p1_node_sum(n3, ev + 18, 2)));
+          n3[k] = p1_cross_pair(c1[(k + 1) % 3], c1[(k + 2) % 3], c2[(k + 1) % 3], c2[(k + 2) % 3]);
+#pragma unroll
+        for (int v = 0; v < 3; ++v) {
+          float2 p[3];
+#pragma unroll
+          for (int k = 0; k < 3; ++k) p[k] = p1_mul(n3[k], ev[12 + 3 * v + k]);
+          zab[iz][v] = p1_norm(p1_mul(zwp[iz], p1_sum3(p[v], p[(v + 1) % 3], p[(v + 2) % 3])));
+        }
+      }
+      if (!in_range) {
+        float t[33];
+        p1_setup64(in, zd, zwd, t);
+#pragma unroll
+        for (int k = 0; k < 21; ++k) ev32[k] = t[k];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) zab[j / 3][j % 3] = make_float2(t[21 + 2 * j], t[22 + 2 * j]);
       }
     }
     // FP32 columns c1, c2 and n3 per vertical node
@@ -342,13 +534,12 @@ __global__ void __launch_bounds__(kP1Threads, 3) cc_p1_kernel(FwdArgs a) {
       cross3(zc[iz], zc[iz] + 3, zc[iz] + 6);
     }
     float cf[14];
-    const bool perq = a.coef_mode == FEI_COEF_PER_POINT;
     if (!perq) {
       double cd[14];
-      ok &= load_coef(a, e, cd);
-      sym = !a.upper || coef_symmetric(cd, cd + 9);
 #pragma unroll
-      for (int k = 0; k < 14; ++k) cf[k] = (float)cd[k];
+      for (int k = 0; k < 14; ++k) cd[k] = in[18 + k];
+      sym = !a.upper || coef_symmetric(cd, cd + 9);
+      ok &= coef_to_f32<14>(cd, cf);
     }
     int st = !ok ? FEI_ERR_NONFINITE : (!sym ? FEI_ERR_INVALID_ARG : 0);
     float A[NSH][NSH], bv[NSH];
@@ -398,23 +589,55 @@ __global__ void __launch_bounds__(kP1Threads, 3) cc_p1_kernel(FwdArgs a) {
         bv[i] = __fadd_rn(bv[i], c[NSH * NSH + i]);
       }
     }
-    float *Ao = reinterpret_cast<float *>(a.A) + out_a(a, item, e, NSH);
+    // the tile's outputs by consecutive threads, as 16-byte values where the
+    // tile's matrices are one aligned range
+    if (tid < nt) a.status[e] = st;
+    __syncthreads();
+    if (flat) {
+      float4 *o4 = reinterpret_cast<float4 *>(tile);
+      float2 *o2 = reinterpret_cast<float2 *>(o4 + kP1Threads * 9);
 #pragma unroll
-    for (int i = 0; i < NSH; ++i)
+      for (int v = 0; v < 9; ++v) {
+        const float *r = &A[0][0] + 4 * v;
+        o4[tid * 9 + v] = st ? make_float4(0.f, 0.f, 0.f, 0.f) : make_float4(r[0], r[1], r[2], r[3]);
+      }
 #pragma unroll
-      for (int j = 0; j < NSH; ++j)
-        if (!a.upper || j >= i) Ao[a_pos(i, j, NSH, a.upper)] = st ? 0.f : A[i][j];
-    float *bo = reinterpret_cast<float *>(a.bv) + out_b(a, item, e, NSH);
+      for (int v = 0; v < 3; ++v) o2[tid * 3 + v] = st ? make_float2(0.f, 0.f) : make_float2(bv[2 * v], bv[2 * v + 1]);
+      __syncthreads();
+      float4 *A4 = reinterpret_cast<float4 *>(reinterpret_cast<float *>(a.A) + base * 36);
+      float2 *b2 = reinterpret_cast<float2 *>(reinterpret_cast<float *>(a.bv) + base * 6);
 #pragma unroll
-    for (int i = 0; i < NSH; ++i) bo[i] = st ? 0.f : bv[i];
-    a.status[e] = st;
+      for (int v = 0; v < 9; ++v)
+        if (tid + v * kP1Threads < nt * 9) A4[tid + v * kP1Threads] = o4[tid + v * kP1Threads];
+#pragma unroll
+      for (int v = 0; v < 3; ++v)
+        if (tid + v * kP1Threads < nt * 3) b2[tid + v * kP1Threads] = o2[tid + v * kP1Threads];
+    } else {
+#pragma unroll
+      for (int i = 0; i < NSH; ++i) {
+#pragma unroll
+        for (int j = 0; j < NSH; ++j) outs[tid * OUT + i * NSH + j] = st ? 0.f : A[i][j];
+        outs[tid * OUT + NSH * NSH + i] = st ? 0.f : bv[i];
+      }
+      __syncthreads();
+      for (int i = tid; i < nt * 36; i += kP1Threads) {
+        const int el = i / 36, k = i - el * 36, r = k / NSH, c = k - r * NSH;
+        if (!a.upper || c >= r)
+          reinterpret_cast<float *>(a.A)[out_a(a, base + el, eid[el], NSH) + a_pos(r, c, NSH, a.upper)] = outs[el * OUT + k];
+      }
+      for (int i = tid; i < nt * 6; i += kP1Threads) {
+        const int el = i / 6, k = i - el * 6;
+        reinterpret_cast<float *>(a.bv)[out_b(a, base + el, eid[el], NSH) + k] = outs[el * OUT + 36 + k];
+      }
+    }
+    __syncthreads();
   }
 }
 
 // p = 1, FP32 path, small batches: eight lanes per element (one per
 // point), so that a batch that fills only part of the GPU (4096 prisms:
 // 32 blocks of the kernel above) is not bound by one thread walking its
-// eight points in turn.  The FP64 work is spread over the lanes (three
+// eight points in turn.  The setup is spread over the lanes (three
 // element-vector components per lane, three lanes per vertical node for
 // the node sums), each lane forms its point's contribution to A_e and b_e
 // in registers, and a butterfly over the eight lanes adds them up.
@@ -425,6 +648,7 @@ __global__ void __launch_bounds__(kP1Threads) cc_p1_small_kernel(FwdArgs a) {
   __shared__ float ttabf[NT][3];
   __shared__ float zf[M], zwf[M];
   __shared__ double zd[M], zwd[M];
+  __shared__ float2 zp[M], zwp[M];
   for (int k = threadIdx.x; k < 4 * NQ * NSH; k += blockDim.x) Gs[k] = a.G32[k];
   if (threadIdx.x < NT) {
     const int t = threadIdx.x;
@@ -441,6 +665,8 @@ __global__ void __launch_bounds__(kP1Threads) cc_p1_small_kernel(FwdArgs a) {
     zwd[iz] = a.znode[2 * iz + 1];
     zf[iz] = (float)zd[iz];
     zwf[iz] = (float)zwd[iz];
+    zp[iz] = split_f64(zd[iz]);
+    zwp[iz] = split_f64(zwd[iz]);
   }
   __syncthreads();
   const int lane = threadIdx.x & 31, g = lane & 7, gbase = lane & 24;
@@ -460,50 +686,60 @@ __global__ void __launch_bounds__(kP1Threads) cc_p1_small_kernel(FwdArgs a) {
     // from global memory (the group's 144 bytes, cached), in FP64
     const double *X = a.geom + 18 * e;
     bool ok = finite64(X[g]) && finite64(X[g + 8]) && (g >= 2 || finite64(X[g + 16]));
-    double evm[3];
-    float evfm[3];
+    float2 evm[3];
+    bool in_range = true;
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
       const int j = g + 8 * r;
-      evm[r] = elem_vec_comp(X, j < 21 ? j : 20);
-      evfm[r] = (float)evm[r];
+      evm[r] = elem_vec_pair(X, j < 21 ? j : 20, &in_range);
     }
+    auto ev2 = [&](int j) {
+      return make_float2(__shfl_sync(0xffffffffu, evm[j / 8].x, gbase + (j & 7)),
+                         __shfl_sync(0xffffffffu, evm[j / 8].y, gbase + (j & 7)));
+    };
+    float2 ev[21];
     float ev32[21];
 #pragma unroll
-    for (int j = 0; j < 21; ++j) ev32[j] = __shfl_sync(0xffffffffu, evfm[j / 8], gbase + (j & 7));
-    auto ev64 = [&](int j) { return __shfl_sync(0xffffffffu, evm[j / 8], gbase + (j & 7)); };
+    for (int j = 0; j < 21; ++j) {
+      ev[j] = ev2(j);
+      ev32[j] = ev[j].x;
+    }
     // node sums: lanes 0..5 of the group, three per vertical node
     float2 zab[M][3];
     {
       const int iz = g < 3 ? 0 : 1, k = g < 6 ? g - 3 * iz : 0;
       const int l1 = gbase + 3 * iz + (k + 1) % 3, l2 = gbase + 3 * iz + (k + 2) % 3;
-      // components k of A1, B1, A2, B2, C, D1, D2 (the shuffles run in all lanes)
-      double e0 = ev64(0), e1 = ev64(1), e2 = ev64(2), e3 = ev64(3), e4 = ev64(4), e5 = ev64(5);
-      double e6 = ev64(6), e7 = ev64(7), e8 = ev64(8), e9 = ev64(9), e10 = ev64(10), e11 = ev64(11);
-      double e12 = ev64(12), e13 = ev64(13), e14 = ev64(14), e15 = ev64(15), e16 = ev64(16), e17 = ev64(17);
-      double e18 = ev64(18), e19 = ev64(19), e20 = ev64(20);
-      const double A1 = k == 0 ? e0 : k == 1 ? e1 : e2, B1 = k == 0 ? e3 : k == 1 ? e4 : e5;
-      const double A2 = k == 0 ? e6 : k == 1 ? e7 : e8, B2 = k == 0 ? e9 : k == 1 ? e10 : e11;
-      const double Cc = k == 0 ? e12 : k == 1 ? e13 : e14, D1 = k == 0 ? e15 : k == 1 ? e16 : e17;
-      const double D2 = k == 0 ? e18 : k == 1 ? e19 : e20;
-      const double z = zd[iz], wz = zwd[iz];
-      const double c1 = fma(z, B1, A1), c2 = fma(z, B2, A2);
-      const double c1a = __shfl_sync(0xffffffffu, c1, l1), c1b = __shfl_sync(0xffffffffu, c1, l2);
-      const double c2a = __shfl_sync(0xffffffffu, c2, l1), c2b = __shfl_sync(0xffffffffu, c2, l2);
-      const double n3 = p1_cross_comp(c1a, c1b, c2a, c2b);
+      auto shfl2 = [](float2 v, int src) {
+        return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
+      };
+      // component k of a vector
+      auto comp = [&](int v) { return k == 0 ? ev[3 * v] : k == 1 ? ev[3 * v + 1] : ev[3 * v + 2]; };
+      const float2 z = zp[iz], wz = zwp[iz];
+      const float2 c1 = p1_column(z, comp(0), comp(1)), c2 = p1_column(z, comp(2), comp(3));
+      const float2 c1a = shfl2(c1, l1), c1b = shfl2(c1, l2), c2a = shfl2(c2, l1), c2b = shfl2(c2, l2);
+      const float2 n3 = p1_cross_pair(c1a, c1b, c2a, c2b);
       // lane k of the node keeps value k, summed as (p_k + p_k+1) + p_k+2
-      const double pa = __dmul_rn(n3, Cc), pb = __dmul_rn(n3, D1), pc = __dmul_rn(n3, D2);
-      const double s_al = __dadd_rn(__dadd_rn(pa, __shfl_sync(0xffffffffu, pa, l1)), __shfl_sync(0xffffffffu, pa, l2));
-      const double s_be = __dadd_rn(__dadd_rn(pb, __shfl_sync(0xffffffffu, pb, l1)), __shfl_sync(0xffffffffu, pb, l2));
-      const double s_ga = __dadd_rn(__dadd_rn(pc, __shfl_sync(0xffffffffu, pc, l1)), __shfl_sync(0xffffffffu, pc, l2));
-      const float2 mine = split_f64(__dmul_rn(wz, k == 0 ? s_al : k == 1 ? s_be : s_ga));
+      float2 sum[3];
+#pragma unroll
+      for (int v = 0; v < 3; ++v) {
+        const float2 p = p1_mul(n3, comp(4 + v)), pa = shfl2(p, l1), pb = shfl2(p, l2);
+        sum[v] = p1_sum3(p, pa, pb);
+      }
+      const float2 mine = p1_norm(p1_mul(wz, k == 0 ? sum[0] : k == 1 ? sum[1] : sum[2]));
 #pragma unroll
       for (int n = 0; n < M; ++n)
 #pragma unroll
-        for (int v = 0; v < 3; ++v) {
-          zab[n][v].x = __shfl_sync(0xffffffffu, mine.x, gbase + 3 * n + v);
-          zab[n][v].y = __shfl_sync(0xffffffffu, mine.y, gbase + 3 * n + v);
-        }
+        for (int v = 0; v < 3; ++v) zab[n][v] = shfl2(mine, gbase + 3 * n + v);
+    }
+#pragma unroll
+    for (int off = 4; off >= 1; off >>= 1) in_range &= __shfl_xor_sync(0xffffffffu, (int)in_range, off) != 0;
+    if (!in_range) {
+      float t[33];
+      p1_setup64(X, zd, zwd, t);
+#pragma unroll
+      for (int k = 0; k < 21; ++k) ev32[k] = t[k];
+#pragma unroll
+      for (int j = 0; j < 6; ++j) zab[j / 3][j % 3] = make_float2(t[21 + 2 * j], t[22 + 2 * j]);
     }
     // coefficients: components g and g + 8 per lane, shared in FP32
     float cf[14];
@@ -611,9 +847,8 @@ fei_status launch_p1(const FwdArgs &a, int64_t grid_work, cudaStream_t s, int64_
     return FEI_OK;
   }
   int64_t blocks = (grid_work + kP1Threads - 1) / kP1Threads;
-  const int64_t cap = grid_cap > 0 ? grid_cap : (a.count ? 152 * 8 : 0);
-  if (cap > 0 && blocks > cap) blocks = cap;
-  if (blocks > 2147483647LL) blocks = 2147483647LL;
+  const int64_t cap = grid_cap > 0 ? grid_cap : 152 * 3;  // resident blocks: the tables are loaded once
+  if (blocks > cap) blocks = cap;
   if (blocks < 1) blocks = 1;
   cc_p1_kernel<<<(unsigned)blocks, kP1Threads, 0, s>>>(a);
   FEI_CUDA_TRY(cudaGetLastError(), "cc_p1_kernel launch");

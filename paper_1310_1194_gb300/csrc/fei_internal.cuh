@@ -96,6 +96,29 @@ __device__ __forceinline__ int64_t out_b(const FwdArgs &a, int64_t k, int64_t e,
   return a.b_off ? a.b_off[e] : (a.out_by_item ? k : e) * s;
 }
 
+// The bucketing of a mixed batch: lists[p - 1][..] of the elements of degree p
+// (in no fixed order), statuses of the elements without a bucket.  The lanes
+// of a warp that share a degree take their places with one atomic (one per
+// element serialises on seven addresses: 400 000 elements 0.2 ms).
+__device__ __forceinline__ void bucket_elements(const int32_t *degree, int64_t n, unsigned avail, int32_t *counts,
+                                                int32_t *lists, int64_t cap, int32_t *status) {
+  const int lane = threadIdx.x & 31;
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  // whole warps run every iteration
+  for (int64_t e0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; e0 < n; e0 += step) {
+    const int64_t e = e0 + lane;
+    const int p = e < n ? degree[e] : 0;
+    const bool ok = p >= 1 && p <= kPMax && ((avail >> p) & 1u);
+    const unsigned same = __match_any_sync(0xffffffffu, ok ? p : 0);
+    const int leader = __ffs(same) - 1;
+    int pos = 0;
+    if (ok && lane == leader) pos = atomicAdd(&counts[p], __popc(same));
+    pos = __shfl_sync(0xffffffffu, pos, leader) + __popc(same & ((1u << lane) - 1u));
+    if (ok) lists[(int64_t)(p - 1) * cap + pos] = (int32_t)e;
+    else if (e < n && status) status[e] = FEI_ERR_INVALID_DEGREE;
+  }
+}
+
 struct BwdArgs {
   int64_t n_work;
   const int32_t *count;

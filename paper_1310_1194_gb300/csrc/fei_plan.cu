@@ -149,15 +149,7 @@ fei_status launch_degree(const fei_plan *pl, int p, int variant, int64_t grid_ca
 
 __global__ void plan_bucket_kernel(const int32_t *degree, int64_t n, unsigned avail, int32_t *counts,
                                    int32_t *lists, int64_t cap, int32_t *status) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    const int p = degree[e];
-    if (p >= 1 && p <= kPMax && ((avail >> p) & 1u)) {
-      const int pos = atomicAdd(&counts[p], 1);
-      lists[(int64_t)(p - 1) * cap + pos] = (int32_t)e;
-    } else {
-      status[e] = FEI_ERR_INVALID_DEGREE;
-    }
-  }
+  bucket_elements(degree, n, avail, counts, lists, cap, status);
 }
 
 fei_status enqueue_bucketing(const fei_plan *pl, const fei_batch *b, int32_t *st, cudaStream_t s) {

@@ -160,3 +160,34 @@ def test_adjoint_counts_and_lists(p, precision, tol_elem, tol_rec):
                                      precision=precision)
     for x, y in zip(one, full):
         assert torch.equal(x[0], y[idx[2]])
+
+
+def test_p1_kernels_agree_in_and_out_of_the_pair_range():
+    """p = 1: the one-thread kernel (above 16384 elements) and the eight-lane
+    kernel give the same bits, tiles with a ragged end, elements of a list,
+    and elements whose vertex differences are outside the FP32 pairs' range
+    (an axis scaled to 1e-19) included; sampled elements against the oracle."""
+    n = 16384 + 77
+    w = inputs.workload("p1m", n_max=n)
+    w = take(w, np.arange(n))
+    odd = np.arange(5, n, 1000)
+    w["geom"][odd] *= np.array([1e-19, 1e9, 1e9])
+    A, b, st = run(w, "fp32", p=1)
+    assert not st.any()
+    idx = np.r_[0, 5, 127, 128, 1005, 16389, n - 1]
+    As, bs, _ = run(take(w, idx), "fp32", p=1)
+    assert np.array_equal(A.reshape(n, 36)[idx], As.reshape(-1, 36))
+    assert np.array_equal(b.reshape(n, 6)[idx], bs.reshape(-1, 6))
+    sub = take(w, idx)
+    Ao, bo, so, _ = oracle.integrate(*(sub[k] for k in ("geom", "K", "b", "c", "f")), p=1)
+    off, sizes = np.arange(len(idx)) * 36, np.full(len(idx), 36)
+    assert not so.any() and per_elem_err(As, Ao, off, sizes).max() < 1e-5
+    assert per_elem_err(bs, bo, off // 6, sizes // 6).max() < 1e-5
+    # as every second element of a list of 2 n elements of degrees 1 and 2
+    m = 200
+    both = {k: np.repeat(w[k][:m], 2, axis=0) for k in w}
+    degree = np.tile(np.array([2, 1], dtype=np.int32), m)
+    Al, bl, sl = run(both, "fp32", degree=degree)
+    at = np.r_[0, np.cumsum(np.where(degree == 1, 36, 324))]
+    got = np.stack([Al[at[2 * i + 1]:at[2 * i + 2]] for i in range(m)])
+    assert np.array_equal(got, A.reshape(n, 36)[:m])
