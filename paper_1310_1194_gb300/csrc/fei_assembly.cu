@@ -19,16 +19,15 @@
 //      rank of l2g_e[j] among them, the same for every private row of the
 //      element: one uint16 rank per local function.  A shared row needs its
 //      own offsets: for each shared local row i, the place of every l2g_e[j]
-//      in row l2g_e[i] (uint16), reached through a per-row slot;
+//      in row l2g_e[i] (uint16), and a record with where the row starts;
 //   5. elements sorted by (degree, colour): the runs of equal (degree,
 //      colour) are the assembly launches, in that order, for both entry
 //      points (so both add the contributions of a shared entry in the same
 //      order); for the fused path, the elements of one degree split into
 //      chunks where a chunk's element matrices would pass a size cap.
-// Device part (fei_assemble): the shared rows are cleared, then a block
-// per element stores its entries of private rows (the only contribution
-// they get) and adds those of shared rows, one launch per (degree, colour)
-// run.  fei_integrate_assemble integrates the batch chunk by chunk into one
+// Device part (fei_assemble): the shared rows are cleared; the entries of
+// private rows (the only contribution they get) are stored by one launch per
+// degree, those of shared rows added by one launch per (degree, colour) run.  fei_integrate_assemble integrates the batch chunk by chunk into one
 // scratch buffer (one forward launch per chunk, all colours of a degree
 // together) and assembles each chunk from it run by run, so that a batch
 // never needs memory for all of its element matrices at once.
@@ -40,6 +39,13 @@
 #include <vector>
 
 #include "fei_internal.cuh"
+
+// A shared row of one element: local row i of element e (global row g, start
+// base in the values), its columns' places at shoff + so.
+struct SharedRow {
+  int64_t base, so, g;
+  int32_t e, i;
+};
 
 struct fei_assembly {
   int64_t n_elem, n_dof, nnz, n_entries;
@@ -67,10 +73,12 @@ struct fei_assembly {
   int64_t *moff;     // start of element e in A (sum of N_sh^2)
   uint16_t *rank;    // [loff layout] rank of l2g_e[j] among the element's functions
   int16_t *slot;     // [loff layout] shared-row slot of local row i, -1 = private
-  int64_t *shptr;    // [n_elem] start of element e's shared-row offsets in shoff
+  SharedRow *shrow_recs;             // the elements' shared rows in the order of elems
+  std::vector<int64_t> shrow_start;  // [n_elem + 1] first record of elems[k]
   uint16_t *shoff;   // per shared row: the N_sh places of the element's columns
   int32_t *shrows;   // global rows touched by several elements (cleared first)
   int64_t n_shrows;
+  bool has_private[fei::kPMax + 1];  // degrees with rows that one element alone touches
   int32_t *elems;        // elements sorted by (colour, degree)
   int32_t *chunk_count;  // [chunks] element count of each chunk (the forward's device count)
   int64_t *scr_aoff, *scr_boff;  // start of element e in its chunk's scratch
@@ -96,69 +104,120 @@ __global__ void clear_rows_kernel(const int32_t *rows, int64_t n, const int64_t 
   }
 }
 
-// One run of elements of a single degree (s functions each) that share no
-// global function: work unit u is rows [rb part, rb part + rb) of element
-// k = u / units_per_element (a warp per row, lanes over columns), so that a
-// run of few large elements still fills the GPU.
-template <typename T>
-__global__ void assemble_kernel(const int32_t *elems, int64_t n, int s, int rb, const T *A, const int64_t *aoff,
-                                const T *bv, const int64_t *boff, const int64_t *l2g, const int64_t *loff,
-                                const uint16_t *rank, const int16_t *slot, const int64_t *shptr,
-                                const uint16_t *shoff, const int64_t *row_ptr, T *values, T *rhs) {
-  __shared__ int64_t rstart[nsh_of(kPMax)];
-  __shared__ int16_t sl[nsh_of(kPMax)];
-  __shared__ uint16_t rk[nsh_of(kPMax)];
-  const int upe = (s + rb - 1) / rb;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int64_t u = blockIdx.x; u < n * upe; u += gridDim.x) {
-    const int64_t k = u / upe;
-    const int i0 = (int)(u - k * upe) * rb;
-    const int nr = s - i0 < rb ? s - i0 : rb;
+// The private rows of elements of one degree, any colours: every entry has
+// this one contribution, so it is stored.  A block per element runs over the
+// matrix as one range of consecutive values, several loads in flight per
+// thread; blocks of other elements hide the chain of index loads.  Bound by
+// HBM: at p = 4, 36 000 prisms, A_e is read and the values written once.
+template <typename T, int P>
+__global__ void __launch_bounds__(256) assemble_private_kernel(const int32_t *elems, int64_t n, const T *A,
+                                                               const int64_t *aoff, const T *bv, const int64_t *boff,
+                                                               const int64_t *l2g, const int64_t *loff,
+                                                               const uint16_t *rank, const int16_t *slot,
+                                                               const int64_t *row_ptr, T *values, T *rhs) {
+  constexpr int S = nsh_of(P), U = 8;
+  __shared__ int64_t rstart[S];  // start of the row in values, -1 for a shared row
+  __shared__ uint16_t rk[S];
+  for (int64_t k = blockIdx.x; k < n; k += gridDim.x) {
     const int e = elems[k];
-    const int64_t lo = loff[e];
-    __syncthreads();  // the previous unit's row data are no longer read
-    for (int j = threadIdx.x; j < s; j += blockDim.x) rk[j] = rank[lo + j];
-    for (int t = threadIdx.x; t < nr; t += blockDim.x) {
-      const int64_t g = l2g[lo + i0 + t];
-      rstart[t] = row_ptr[g];
-      sl[t] = slot[lo + i0 + t];
-      rhs[g] += bv[boff[e] + i0 + t];
+    const int64_t lo = loff[e], bo = boff[e];
+    const T *Ae = A + aoff[e];
+    __syncthreads();  // the previous element's row data are no longer read
+    for (int j = threadIdx.x; j < S; j += 256) {
+      rk[j] = rank[lo + j];
+      const bool own = slot[lo + j] < 0;
+      const int64_t g = l2g[lo + j];
+      rstart[j] = own ? row_ptr[g] : -1;
+      if (own) rhs[g] += bv[bo + j];
     }
     __syncthreads();
-    const T *Ae = A + aoff[e];
-    const uint16_t *so = shoff + shptr[e];
-    for (int t = warp; t < nr; t += nw) {
-      const int i = i0 + t, q = sl[t];
-      const int64_t base = rstart[t];
-      const T *Ai = Ae + (int64_t)i * s;
-      if (q < 0) {
-        for (int j = lane; j < s; j += 32) values[base + rk[j]] = Ai[j];  // a private row: its only contribution
-      } else {
-        const uint16_t *o = so + q * s;
-        for (int j = lane; j < s; j += 32) values[base + o[j]] += Ai[j];
+    for (int i0 = threadIdx.x; i0 < S * S; i0 += 256 * U) {
+      T v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (i0 + 256 * u < S * S) v[u] = Ae[i0 + 256 * u];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int ij = i0 + 256 * u, i = ij / S, j = ij - i * S;
+        if (ij < S * S) {
+          const int64_t r = rstart[i];
+          if (r >= 0) values[r + rk[j]] = v[u];
+        }
       }
     }
   }
 }
 
-// elems[0 .. n): one run (one degree p)
-template <typename T>
-fei_status launch_assemble(const fei_assembly *as, int p, const int32_t *elems, int64_t n, const void *A,
-                           const int64_t *aoff, const void *bv, const int64_t *boff, void *values, void *rhs,
-                           cudaStream_t s) {
-  if (n <= 0) return FEI_OK;
-  const int sh = nsh_of(p);
-  // rows per work unit: whole elements when the run has enough of them,
-  // else split so that the run gives about 8 units per SM (at least 32 rows)
-  int64_t rb = (n * sh + 152 * 8 - 1) / (152 * 8);
-  rb = rb < 32 ? 32 : (rb > sh ? sh : rb);
-  const int64_t units = n * ((sh + rb - 1) / rb);
-  const int64_t blocks = units < 152 * 16 ? units : 152 * 16;
-  assemble_kernel<T><<<(unsigned)blocks, 256, 0, s>>>(elems, n, sh, (int)rb, (const T *)A, aoff, (const T *)bv, boff,
-                                                      as->l2g, as->loff, as->rank, as->slot, as->shptr, as->shoff,
-                                                      as->row_ptr, (T *)values, (T *)rhs);
+// The shared rows of one run of elements of a single degree that share no
+// global function: their entries are added, a warp per row (p = 1: eight
+// lanes).  The records hold
+// what a row needs, in run order (through element, slot and row tables the
+// chain of dependent loads took three times as long: 20 us a run of 3000
+// elements at p = 4).
+template <typename T, int P>
+__global__ void __launch_bounds__(256) assemble_shared_kernel(const SharedRow *rows, int64_t n, const T *A,
+                                                              const int64_t *aoff, const T *bv, const int64_t *boff,
+                                                              const uint16_t *shoff, T *values, T *rhs) {
+  constexpr int S = nsh_of(P), G = S <= 8 ? 8 : 32, NL = (S + G - 1) / G;
+  const int lane = threadIdx.x % G;
+  for (int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G; k < n;
+       k += (int64_t)gridDim.x * (blockDim.x / G)) {
+    const SharedRow r = rows[k];
+    const T *Ai = A + aoff[r.e] + (int64_t)r.i * S;
+    const uint16_t *o = shoff + r.so;
+    T *row = values + r.base;
+    T v[NL];
+    int at[NL];
+#pragma unroll
+    for (int c = 0; c < NL; ++c)
+      if (G * c + lane < S) at[c] = o[G * c + lane], v[c] = Ai[G * c + lane];
+#pragma unroll
+    for (int c = 0; c < NL; ++c)
+      if (G * c + lane < S) v[c] += row[at[c]];
+#pragma unroll
+    for (int c = 0; c < NL; ++c)
+      if (G * c + lane < S) row[at[c]] = v[c];
+    if (lane == 0) rhs[r.g] += bv[boff[r.e] + r.i];
+  }
+}
+
+// Elements elems[k0 .. k1) of one degree p, their matrices and vectors at
+// aoff[e], boff[e]: the private rows of all of them, or the shared rows of
+// one run (no two elements share a function).
+template <typename T, int P>
+fei_status launch_assemble_p(const fei_assembly *as, int64_t k0, int64_t k1, bool shared, const void *A,
+                             const int64_t *aoff, const void *bv, const int64_t *boff, void *values, void *rhs,
+                             cudaStream_t s) {
+  if (shared) {
+    const int64_t r0 = as->shrow_start[k0], n = as->shrow_start[k1] - r0;
+    if (n == 0) return FEI_OK;
+    const int64_t per = P == 1 ? 32 : 8, blocks = (n + per - 1) / per;  // rows per block
+    assemble_shared_kernel<T, P><<<(unsigned)(blocks < 152 * 64 ? blocks : 152 * 64), 256, 0, s>>>(
+        as->shrow_recs + r0, n, (const T *)A, aoff, (const T *)bv, boff, as->shoff, (T *)values, (T *)rhs);
+  } else {
+    const int64_t n = k1 - k0;
+    assemble_private_kernel<T, P><<<(unsigned)(n < 152 * 32 ? n : 152 * 32), 256, 0, s>>>(
+        as->elems + k0, n, (const T *)A, aoff, (const T *)bv, boff, as->l2g, as->loff, as->rank, as->slot, as->row_ptr,
+        (T *)values, (T *)rhs);
+  }
   FEI_CUDA_TRY(cudaGetLastError(), "assemble_kernel launch");
   return debug_check(s, "assemble_kernel");
+}
+template <typename T>
+fei_status launch_assemble(const fei_assembly *as, int p, int64_t k0, int64_t k1, bool shared, const void *A,
+                           const int64_t *aoff, const void *bv, const int64_t *boff, void *values, void *rhs,
+                           cudaStream_t s) {
+  if (k1 <= k0 || (!shared && !as->has_private[p])) return FEI_OK;
+  switch (p) {
+    case 1: return launch_assemble_p<T, 1>(as, k0, k1, shared, A, aoff, bv, boff, values, rhs, s);
+    case 2: return launch_assemble_p<T, 2>(as, k0, k1, shared, A, aoff, bv, boff, values, rhs, s);
+    case 3: return launch_assemble_p<T, 3>(as, k0, k1, shared, A, aoff, bv, boff, values, rhs, s);
+    case 4: return launch_assemble_p<T, 4>(as, k0, k1, shared, A, aoff, bv, boff, values, rhs, s);
+    case 5: return launch_assemble_p<T, 5>(as, k0, k1, shared, A, aoff, bv, boff, values, rhs, s);
+    case 6: return launch_assemble_p<T, 6>(as, k0, k1, shared, A, aoff, bv, boff, values, rhs, s);
+    case 7: return launch_assemble_p<T, 7>(as, k0, k1, shared, A, aoff, bv, boff, values, rhs, s);
+  }
+  return set_error(FEI_ERR_INVALID_DEGREE, "degree %d outside 1..7", p);
 }
 
 // values of the shared rows and the whole rhs set to zero (private rows are
@@ -183,7 +242,7 @@ void free_device(fei_assembly *as) {
   cudaFree(as->moff);
   cudaFree(as->rank);
   cudaFree(as->slot);
-  cudaFree(as->shptr);
+  cudaFree(as->shrow_recs);
   cudaFree(as->shoff);
   cudaFree(as->shrows);
   cudaFree(as->elems);
@@ -318,6 +377,7 @@ fei_status build(fei_assembly *as, const int64_t *l2g) {
   }
   // 4. scatter map: ranks (computed above), slots of shared rows and
   // their offsets, and the list of shared rows
+  for (bool &own : as->has_private) own = false;
   std::vector<int16_t> slot(loff[n], -1);
   std::vector<int64_t> shptr(n + 1, 0);
   for (int64_t e = 0; e < n; ++e) {
@@ -326,6 +386,7 @@ fei_status build(fei_assembly *as, const int64_t *l2g) {
     for (int64_t i = 0; i < s; ++i) {
       const int64_t r = l2g[loff[e] + i];
       if (inc_ptr[r + 1] - inc_ptr[r] > 1) slot[loff[e] + i] = (int16_t)q++;
+      else as->has_private[as->degree_h[e]] = true;
     }
     shptr[e + 1] = shptr[e] + q * s;
   }
@@ -360,6 +421,18 @@ fei_status build(fei_assembly *as, const int64_t *l2g) {
       as->run_degree.push_back(as->degree_h[elems[k - 1]]);
       as->run_start.push_back(k);
     }
+  std::vector<SharedRow> recs;
+  as->shrow_start.assign(1, 0);
+  for (int64_t k = 0; k < n; ++k) {
+    const int32_t e = elems[k];
+    const int64_t s = loff[e + 1] - loff[e];
+    for (int64_t i = 0; i < s; ++i) {
+      const int16_t q = slot[loff[e] + i];
+      const int64_t g = l2g[loff[e] + i];
+      if (q >= 0) recs.push_back({row_ptr[g], shptr[e] + q * s, g, e, (int32_t)i});
+    }
+    as->shrow_start.push_back((int64_t)recs.size());
+  }
   std::vector<int64_t> scr_aoff(n), scr_boff(n);
   as->chunks.clear();
   as->max_chunk_a = as->max_chunk_b = 0;
@@ -399,7 +472,7 @@ fei_status build(fei_assembly *as, const int64_t *l2g) {
   if ((st = upload(&as->moff, moff.data(), moff.size()))) return st;
   if ((st = upload(&as->rank, rank.data(), rank.size()))) return st;
   if ((st = upload(&as->slot, slot.data(), slot.size()))) return st;
-  if ((st = upload(&as->shptr, shptr.data(), shptr.size()))) return st;
+  if ((st = upload(&as->shrow_recs, recs.data(), recs.size()))) return st;
   if ((st = upload(&as->shoff, shoff.data(), shoff.size()))) return st;
   if ((st = upload(&as->shrows, shrows.data(), shrows.size()))) return st;
   if ((st = upload(&as->elems, elems.data(), elems.size()))) return st;
@@ -532,14 +605,21 @@ extern "C" fei_status fei_assemble(fei_assembly_t as, fei_precision prec, const 
   if (!A || !b || !values || !rhs) return set_error(FEI_ERR_INVALID_ARG, "A, b, values and rhs are required");
   cudaStream_t s = (cudaStream_t)stream;
   if ((st = clear_outputs(as, vb, values, rhs, s))) return st;
-  for (size_t r = 0; r + 1 < as->run_start.size(); ++r) {
-    const int64_t k0 = as->run_start[r], k1 = as->run_start[r + 1];
-    const int p = as->run_degree[r];
-    st = vb == 8 ? launch_assemble<double>(as, p, as->elems + k0, k1 - k0, A, as->moff, b, as->loff, values, rhs, s)
-                 : launch_assemble<float>(as, p, as->elems + k0, k1 - k0, A, as->moff, b, as->loff, values, rhs, s);
-    if (st) return st;
+  auto add = [&](int p, int64_t k0, int64_t k1, bool shared) {
+    return vb == 8 ? launch_assemble<double>(as, p, k0, k1, shared, A, as->moff, b, as->loff, values,
+                                             rhs, s)
+                   : launch_assemble<float>(as, p, k0, k1, shared, A, as->moff, b, as->loff, values,
+                                            rhs, s);
+  };
+  const size_t runs = as->run_degree.size();
+  for (size_t r = 0; r < runs && !st;) {
+    // the runs of one degree: their private rows together, then run by run
+    size_t r1 = r;
+    while (r1 < runs && as->run_degree[r1] == as->run_degree[r]) ++r1;
+    st = add(as->run_degree[r], as->run_start[r], as->run_start[r1], false);
+    for (; r < r1 && !st; ++r) st = add(as->run_degree[r], as->run_start[r], as->run_start[r + 1], true);
   }
-  return FEI_OK;
+  return st;
 }
 
 extern "C" fei_status fei_integrate_assemble(fei_assembly_t as, const fei_reference_t *refs, int nrefs,
@@ -603,17 +683,19 @@ extern "C" fei_status fei_integrate_assemble(fei_assembly_t as, const fei_refere
     a.b_off = nullptr;
     a.out_by_item = 1;  // the chunk's matrices in list order: scr_aoff / scr_boff
     if ((st = launch_forward(ch.degree, prec, r, a, ch.n, s))) return st;
-    // the chunk's part of each (degree, colour) run, one launch each
+    // the chunk's private rows, then the shared rows of its part of each
+    // (degree, colour) run
+    auto add = [&](int64_t k0, int64_t k1, bool shared) {
+      return vb == 8 ? launch_assemble<double>(as, ch.degree, k0, k1, shared, as->scratch_A,
+                                               as->scr_aoff, as->scratch_b, as->scr_boff, values, rhs, s)
+                     : launch_assemble<float>(as, ch.degree, k0, k1, shared, as->scratch_A,
+                                              as->scr_aoff, as->scratch_b, as->scr_boff, values, rhs, s);
+    };
     const int64_t c0 = ch.start, c1 = ch.start + ch.n;
+    if ((st = add(c0, c1, false))) return st;
     const size_t r0 = std::upper_bound(as->run_start.begin(), as->run_start.end(), c0) - as->run_start.begin() - 1;
-    for (size_t rr = r0; rr + 1 < as->run_start.size() && as->run_start[rr] < c1; ++rr) {
-      const int64_t k0 = std::max(as->run_start[rr], c0), k1 = std::min(as->run_start[rr + 1], c1);
-      st = vb == 8 ? launch_assemble<double>(as, ch.degree, as->elems + k0, k1 - k0, as->scratch_A, as->scr_aoff,
-                                             as->scratch_b, as->scr_boff, values, rhs, s)
-                   : launch_assemble<float>(as, ch.degree, as->elems + k0, k1 - k0, as->scratch_A, as->scr_aoff,
-                                            as->scratch_b, as->scr_boff, values, rhs, s);
-      if (st) return st;
-    }
+    for (size_t rr = r0; rr + 1 < as->run_start.size() && as->run_start[rr] < c1; ++rr)
+      if ((st = add(std::max(as->run_start[rr], c0), std::min(as->run_start[rr + 1], c1), true))) return st;
   }
   return FEI_OK;
 }
