@@ -33,9 +33,14 @@ namespace fei {
 namespace {
 
 // Threads and blocks per SM: small blocks, several per SM, one to two points a
-// thread; the fastest of the sizes measured (p = 5, 20 000 prisms with
-// per-point fields: 1.43 ms, 224 threads and 3 blocks 1.6, 2 blocks 1.9).  Rows in groups of two m (m = g and
-// M-1-g, alike in size), at p = 7 of one m (shared memory of two blocks).
+// thread.  Rows in groups of two m (m = g and M-1-g, alike in size); at p = 7
+// and p = 5 of one m (the shared memory of two and of five blocks per SM; at
+// p = 4 and 6 the further barriers cost more).  GB300, p = 5, 20 000 prisms with
+// per-point fields: 1.27 ms (groups of two m 1.35; 224 threads and 3 blocks
+// 1.6); the dense adjoint on the tensor cores took 5.0.  The parts, by leaving
+// them out: zeta sums 0.32 ms (their loads of gA: 0.19 ms of HBM time), v sums
+// 0.16, u sums 0.18, the chain 0.31; the rest is barriers and latency (issue
+// 45 % of slots, 15 to 20 warps an SM).
 template <typename T, int P>
 struct AdjCfg {
   static constexpr bool F32 = std::is_same<T, float>::value;
@@ -44,7 +49,7 @@ struct AdjCfg {
   static constexpr int MINB = F32 ? (P <= 2 ? 24 : P == 3 ? 12 : P == 4 ? 6 : P == 5 ? 5 : 2)
                                   : (P <= 2 ? 8 : P == 3 ? 4 : P == 4 ? 2 : 1);
   static constexpr int NW = NTH / 32;
-  static constexpr int GM = P == 7 ? 1 : 2, NG = GM == 1 ? M : (M + 1) / 2;
+  static constexpr int GM = P == 7 || P == 5 ? 1 : 2, NG = GM == 1 ? M : (M + 1) / 2;
   static constexpr int RM = GM == 1 ? M : M + 1;  // most rows of a group
   static constexpr int NE = (M + 1) / 2, NP = (M + 1) / 2;  // NP: pairs (m', M-1-m')
   // Y [row][t'][l] of 4 values (LL, L'L', LL', L'L); the stride of t' an odd
