@@ -70,58 +70,51 @@ def tc_hw_flops(p, precision="tc_f16x3"):
     return 3 * 2 * s * npad * kpad
 
 
+# multiply-adds and additions of the zeta sums per pair (t, t') (products of
+# two Legendre factors in the discrete Legendre basis of the nodes, zero terms
+# left out), by M = p + 1
+ZETA_TERMS = {2: (7, 2), 3: (22, 6), 4: (50, 12), 5: (97, 20), 6: (165, 30), 7: (262, 42), 8: (388, 56)}
+
+
 def sf_flops_per_element(p):
-    """Flops per element of the sum-factorised kernel (M = p+1 nodes per
-    direction, T = (p+1)(p+2)/2 triangle functions, 21 pairs of gradient
-    terms, 4 pairs of zeta factors): per pair the u sum M^3 (M + 2 M^2) and
-    the v sum T^2 M (1 + 2 M), the zeta sum 4 T^2 M (M + 2 M^2), the load
-    vector 2 (M^4 + M^2 T + N_sh M) and the geometry 220 N_q."""
+    """Flops per element of the sum-factorised kernels (M = p+1 nodes per
+    direction, T = (p+1)(p+2)/2 triangle functions): the zeta transform of 13
+    operators, their u sums over half the nodes, the v sums of 9 combinations
+    (9 T M^3 + 6 T^2 M^2 multiply-adds), the zeta sums per pair of triangle
+    functions, the load vector 2 (M^4 + M^2 T + N_sh M) and the geometry
+    220 N_q."""
     M, T = p + 1, (p + 1) * (p + 2) // 2
-    TT = T * T
-    pairs = 21 * (M ** 3 * (M + 2 * M * M) + TT * M * (1 + 2 * M))
-    return pairs + 4 * TT * M * (M + 2 * M * M) + 2 * (M ** 4 + M * M * T + nsh(p) * M) + 220 * nq(p)
+    fma, add = ZETA_TERMS[M]
+    return (13 * M ** 3 * (M + 2) + 13 * M ** 5 + 2 * (9 * T * M ** 3 + 6 * T * T * M * M) + T * T * (2 * fma + add)
+            + 2 * (M ** 4 + M * M * T + nsh(p) * M) + 220 * nq(p))
+
+
+def runs_sum_factorised(d, precision):
+    """Whether degree d runs the sum-factorised kernel under the precision."""
+    return d >= 2 if precision in ("sf_fp32", "fp32", "fp64") else False
 
 
 def kernel_flops(counts, precision):
     """Flops one step's kernels do for the per-degree counts: the sum-
-    factorised kernel's own count at p >= 3 under sf_fp32, the dense
-    contraction's count otherwise."""
-    return sum(int(counts[d]) * (sf_flops_per_element(d) if (precision == "sf_fp32" and d >= 3)
+    factorised kernels' own count where they run, the dense contraction's
+    count otherwise."""
+    return sum(int(counts[d]) * (sf_flops_per_element(d) if runs_sum_factorised(d, precision)
                                  else flops_per_element(d)) for d in range(1, 8))
 
 
-def fp64_pipe_ops_per_element(p):
-    """FP64-pipe instructions per element of the FP32 path at p <= 2: the 21
-    element-vector components (3 adds, a multiply, a conversion each), per
-    vertical node 36 (the columns c1, c2: 6; n3: 6; n3.C, n3.D1, n3.D2: 9;
-    the w_z products: 3; three FP32-pair splits: 12) and the 14 coefficient
-    conversions."""
-    return 21 * 5 + 36 * (p + 1) + 14
-
-
 def bwd_flops_per_element(p):
-    """Algorithmic flops of the adjoint per element: W = gA G^T (8 N_sh^2
-    N_q), dL/dDt = G_q W_q (32 N_sh N_q), the load-vector adjoint (2 N_sh
-    N_q) and the per-point chain to the coefficients and vertices (about
+    """Flops of the general adjoint per element: the forward's sums in
+    reverse and the per-point chain to the coefficients and vertices (about
     600 flops per point)."""
-    s, q = nsh(p), nq(p)
-    return 8 * s * s * q + 34 * s * q + 600 * q
-
-
-def adj_tc_hw_flops(p):
-    """Issued tensor flops of the tensor-core adjoint per element: three
-    products of M = 128-row tiles of (q, b) (ceil(4 N_q / 128) of them),
-    N = N_sh padded to 16 and K = N_sh padded to 32."""
-    s, q = nsh(p), nq(p)
-    return 3 * 2 * ((4 * q + 127) // 128) * 128 * ((s + 15) // 16 * 16) * ((s + 31) // 32 * 32)
+    return sf_flops_per_element(p) + 600 * nq(p)
 
 
 def quad_bwd_flops_per_element(p):
-    """Algorithmic flops of the quadratic-loss adjoint per element: v_q =
-    G_q u (8 N_sh N_q), the outer products (16 N_q) and the per-point chain
-    (about 600 flops per point)."""
-    s, q = nsh(p), nq(p)
-    return 8 * s * q + 616 * q
+    """Flops of the quadratic-loss adjoint per element: v_q by three
+    one-dimensional sums, the outer products (16 N_q) and the per-point
+    chain (about 600 flops per point)."""
+    M = p + 1
+    return 4 * nsh(p) * M + 6 * (nsh(p) + nq(p)) * M + 616 * nq(p)
 
 
 def bytes_per_element(p, out_bytes, per_qp=False, upper=False):
@@ -375,27 +368,14 @@ def roofline_of(dom, counts, precision, peaks, peak_src, live, Bts, ms_all, p, n
         f64_peak = 152 * 2 * 2 * sm_max * 1e6 / 1e12
     if not f32_peak:
         f32_peak = 152 * 128 * 2 * sm_max * 1e6 / 1e12
-    if low_p and precision == "fp64":
-        # the FP64 path at p <= 2: every flop in FP64
-        bound, peak, unit, achieved = "alu", f64_peak, "TFLOP/s", F / (ms * 1e-3) / 1e12
-        peak_note = f64_note
-        hw = {"hbm_gbs": Bts / (ms * 1e-3) / 1e9, "hbm_frac": Bts / (ms * 1e-3) / 1e9 / peaks["hbm_gbs"],
-              "hbm_peak_gbs": peaks["hbm_gbs"]}
-    elif low_p:
-        # p <= 2 on the FP32 path: a few kflops per element against 0.4-0.6 KB
-        # of traffic, but reading the FP64 inputs needs FP64 work, and at
-        # GB300's FP64 rate (1/64 of FP32) that, not HBM, binds.  The work is
-        # counted in FP64-pipe instructions per element (the element vectors:
-        # 21 x (3 adds, a multiply, a conversion); per vertical node the
-        # columns, n3 and its three dot products, w_z and the FP32-pair
-        # splits: 36; the 14 coefficient conversions) against the measured
-        # FP64 FMA instruction rate (half the FP64 flop peak)
-        ops = sum(int(counts[d]) * fp64_pipe_ops_per_element(d) for d in range(1, 3))
-        bound, peak, unit, achieved = "alu", f64_peak / 2, "Tinst/s", ops / (ms * 1e-3) / 1e12
-        peak_note = f64_note + " / 2: FP64 pipe instructions (the FP64 input work binds before HBM)"
-        hw = {"hbm_gbs": Bts / (ms * 1e-3) / 1e9, "hbm_frac": Bts / (ms * 1e-3) / 1e9 / peaks["hbm_gbs"],
-              "hbm_peak_gbs": peaks["hbm_gbs"], "fp64_pipe_ops_per_element": {
-                  str(d): fp64_pipe_ops_per_element(d) for d in range(1, 3) if counts[d]}}
+    if "adjoint" in dom["kernel"]:
+        # the adjoints' own flops (the chain included) on the FP32 or FP64 pipe
+        bound, unit, achieved = "alu", "TFLOP/s", F / (ms * 1e-3) / 1e12
+        peak, peak_note = (f64_peak, f64_note) if precision == "fp64" else (f32_peak, f32_note)
+    elif low_p and p == 1 and precision != "fp64":
+        # p = 1 on the FP32 path: 4 kflops against 0.43 KB an element
+        bound, peak, unit, achieved = "hbm", peaks["hbm_gbs"], "GB/s", Bts / (ms * 1e-3) / 1e9
+        peak_note = f"HBM copy ({peak_src})"
     elif precision in ("tc_f16x3", "tc_3xtf32"):
         # every algorithmic multiply-add is three tensor products (hi*hi,
         # hi*lo, lo*hi), so the peak for algorithmic flops is a third of the
@@ -410,31 +390,25 @@ def roofline_of(dom, counts, precision, peaks, peak_src, live, Bts, ms_all, p, n
             tpeak, tnote = peaks["bf16_tflops"] * 1.1 / 2.25, f"TF32: bf16 peak ({peak_src}) x nominal 1.1/2.25"
         bound, peak, unit, achieved = "tensor", tpeak / 3, "TFLOP/s", F / (ms * 1e-3) / 1e12
         peak_note = tnote + " / 3"
-        if dom["kernel"].startswith("adjoint"):
-            hwF = sum(int(counts[d]) * adj_tc_hw_flops(d) for d in range(3, 6))
-            hw_note = ("issued tcgen05 flops of W^T: 3 products x 2 x 128-row tiles of (q, b) x N_sh pad 16 x "
-                       "N_sh pad 32; the time includes the FP32 chain kernel")
-        else:
-            hwF = sum(int(counts[d]) * tc_hw_flops(d, precision) for d in range(3, 8))
-            hw_note = "issued tcgen05 flops: 3 products x 2 x 128-row tiles x N_pad x 4 N_q"
+        hwF = sum(int(counts[d]) * tc_hw_flops(d, precision) for d in range(3, 8))
+        hw_note = "issued tcgen05 flops: 3 products x 2 x 128-row tiles x N_pad x 4 N_q"
         hw = {"tensor_tflops": hwF / (ms * 1e-3) / 1e12,
               "frac_of_tensor_peak": hwF / (ms * 1e-3) / 1e12 / tpeak,
               "note": hw_note}
-    elif precision == "sf_fp32":
-        # the sum-factorised kernel does its own, smaller flop count on the
-        # FP32 FMA pipe; the dense contraction's count over the same time is
-        # reported beside it as the equivalent rate
+    elif any(counts[d] and runs_sum_factorised(d, precision) for d in range(1, 8)):
+        # the sum-factorised kernels do their own, smaller flop count on the
+        # FP32 or FP64 FMA pipe; the dense contraction's count over the same
+        # time is reported beside it as the equivalent rate
         Fk = kernel_flops(counts, precision)
-        bound, peak, unit, achieved = "alu", f32_peak, "TFLOP/s", Fk / (ms * 1e-3) / 1e12
-        peak_note = f32_note + " (sum-factorised flop count)"
+        bound, unit, achieved = "alu", "TFLOP/s", Fk / (ms * 1e-3) / 1e12
+        peak, peak_note = (f64_peak, f64_note) if precision == "fp64" else (f32_peak, f32_note)
+        peak_note += " (sum-factorised flop count)"
         hw = {"dense_equivalent_tflops": F / (ms * 1e-3) / 1e12,
-              "note": "dense contraction flops (8 N_sh^2 N_q + ...) over the same time"}
-    elif precision == "fp32":
-        bound, peak, unit, achieved = "alu", f32_peak, "TFLOP/s", F / (ms * 1e-3) / 1e12
-        peak_note = f32_note
+              "note": "dense contraction flops (8 N_sh^2 N_q + ...) over the same time",
+              "hbm_frac": Bts / (ms * 1e-3) / 1e9 / peaks["hbm_gbs"]}
     else:
-        bound, peak, unit, achieved = "alu", f64_peak, "TFLOP/s", F / (ms * 1e-3) / 1e12
-        peak_note = f64_note
+        bound, unit, achieved = "alu", "TFLOP/s", F / (ms * 1e-3) / 1e12
+        peak, peak_note = (f64_peak, f64_note) if precision == "fp64" else (f32_peak, f32_note)
     traffic = None
     if dom["kernel"] == "forward" and p is not None and p >= 3 and precision in ("tc_f16x3", "sf_fp32"):
         traffic = measured_traffic("tc_forward_kernel" if precision == "tc_f16x3" else "sf_forward_kernel", p, n)
@@ -444,8 +418,6 @@ def roofline_of(dom, counts, precision, peaks, peak_src, live, Bts, ms_all, p, n
          "hardware": hw}
     if "fwd_ms" in dom:
         r["forward_ms"] = dom["fwd_ms"]
-    if "fp32_adjoint_ms" in dom:
-        r["fp32_cuda_core_adjoint_ms"] = dom["fp32_adjoint_ms"]
     if "adjoint_ms" in dom:
         r["adjoint_ms"] = dom["adjoint_ms"]
         r["adjoint"] = "quadratic loss (gA never formed)"
@@ -488,10 +460,10 @@ def run_workload(name, args, ctx, headline):
 
     precision = args.precision if headline else None
     if precision is None:
-        # the fastest path within 1e-6 of the oracle: the FP32 kernels at
-        # p <= 2, the split tensor-core kernel at p = 3, 4, the sum-factorised
-        # kernel at p = 5..7, and per degree the tuner's pick for a mixed batch
-        precision = "auto" if p is None else "fp32" if p <= 2 else "tc_f16x3" if p <= 4 else "sf_fp32"
+        # the fastest path within 1e-6 of the oracle: the FP32 kernels (p = 1:
+        # a kernel of its own; p >= 2: the sum-factorised kernel), and per
+        # degree the tuner's pick for a mixed batch
+        precision = "auto" if p is None else "fp32" if p <= 2 else "sf_fp32"
     layout = api.fei_plan_offsets(deg, upper) if deg is not None else api.uniform_layout(n, p, upper)
     refs = [api.fei_reference_create(d) for d in ([p] if p is not None else range(1, 8))]
     out_dtype = torch.float64 if precision == "fp64" else torch.float32
@@ -521,9 +493,7 @@ def run_workload(name, args, ctx, headline):
             grads = ((uu[:, :, None] * uu[:, None, :]).reshape(-1).to(torch.float32), (-u).to(torch.float32))
         else:
             grads = (u,)
-    # the general adjoint: W = gA G^T on the tensor cores (split fp16) at a
-    # uniform degree 3..5, else the FP32 CUDA-core adjoint
-    bwd_prec = "tc_f16x3" if (grads is not None and len(grads) == 2 and deg is None and p in (3, 4, 5)) else "fp32"
+    bwd_prec = "fp32"  # the FP32 adjoint (sum-factorised at every degree)
 
     def step(prec=precision, outs=(A, bv, st), mid=None, bprec=None):
         if plan is not None and prec == precision:
@@ -622,31 +592,17 @@ def run_workload(name, args, ctx, headline):
         bwd_ms = statistics.median([mids[k].elapsed_time(evs[k][1]) for k in range(steps)])
         fwd_ms = statistics.median([evs[k][0].elapsed_time(mids[k]) for k in range(steps)])
         if len(grads) == 2:
-            kname = ("adjoint (tensor-core W^T = G gA^T in split fp16, FP32 chain)" if bwd_prec == "tc_f16x3"
-                     else "adjoint (FP32 CUDA-core contraction, FP32 chain)")
-            dom = {"kernel": kname, "ms": bwd_ms, "F": n * bwd_flops_per_element(p), "precision": bwd_prec,
-                   "counts": counts, "fwd_ms": fwd_ms}
-            if bwd_prec == "tc_f16x3" and rank == 0:
-                # the FP32 CUDA-core adjoint on the same cotangents, for comparison
-                tb = []
-                for k in range(min(steps, 3)):
-                    e0, e1, e2 = (torch.cuda.Event(enable_timing=True) for _ in range(3))
-                    flush.fill_(float(k))
-                    e0.record(stream)
-                    step(mid=e1, bprec="fp32")
-                    e2.record(stream)
-                    torch.cuda.synchronize()
-                    tb.append(e1.elapsed_time(e2))
-                dom["fp32_adjoint_ms"] = statistics.median(tb)
+            dom = {"kernel": "adjoint (sum-factorised, FP32 chain)", "ms": bwd_ms, "F": n * bwd_flops_per_element(p),
+                   "precision": bwd_prec, "counts": counts, "fwd_ms": fwd_ms}
         elif bwd_ms > fwd_ms:
-            dom = {"kernel": "quadratic-loss adjoint (fp32 G u, fp64 chain)", "ms": bwd_ms,
+            dom = {"kernel": "quadratic-loss adjoint (sum-factorised v, FP32 chain)", "ms": bwd_ms,
                    "F": n * quad_bwd_flops_per_element(p), "precision": "fp32", "counts": counts, "fwd_ms": fwd_ms}
         else:
             dom = {"kernel": "forward", "ms": fwd_ms, "F": F, "precision": precision, "counts": counts,
                    "adjoint_ms": bwd_ms}
     roofline = roofline_of(dom, dom["counts"], dom["precision"], peaks, peak_src, live, Bts, ms, p, n, per_qp)
     if plan is not None:
-        step_flops = sum(int(counts[d]) * (sf_flops_per_element(d) if prec_of[d] == "sf_fp32" else
+        step_flops = sum(int(counts[d]) * (sf_flops_per_element(d) if runs_sum_factorised(d, prec_of[d]) else
                                            flops_per_element(d)) for d in range(1, 8) if counts[d])
     else:
         step_flops = kernel_flops(counts, precision)
@@ -698,14 +654,11 @@ def run_workload(name, args, ctx, headline):
             del A32, b32, st32
 
     # the other paths on the same batch (time, roofline and error): the
-    # other split of the tensor-core contraction for the headline (fp16 or
-    # TF32 operands), and both splits for the p = 7 workload, where the
-    # sum-factorised kernel is the timed path
+    # splits of the tensor-core contraction (fp16 or TF32 operands) for the
+    # headline and for the p = 7 workload
     alts = []
     if rank == 0 and p is not None and p >= 3 and grads is None:
-        if headline and precision in ("tc_f16x3", "tc_3xtf32"):
-            alts = ["tc_3xtf32" if precision == "tc_f16x3" else "tc_f16x3"]
-        elif name == "p7":
+        if headline or name == "p7":
             alts = [x for x in ("tc_f16x3", "tc_3xtf32", "sf_fp32") if x != precision]
     other = {}
     for alt in alts:
@@ -730,7 +683,8 @@ def run_workload(name, args, ctx, headline):
         if ref is not None:
             other[alt]["rel_err_vs_oracle"] = errors_vs_oracle(Aa, ba, sa, ref, n_s, p if upper else None)
         del Aa, ba, sa
-    alt_tc = other.get("tc_3xtf32" if precision == "tc_f16x3" else "tc_f16x3") if headline else None
+    alt_tc = other.get("tc_3xtf32" if precision == "tc_f16x3" else "tc_f16x3") if (
+        headline and precision in ("tc_f16x3", "tc_3xtf32")) else None
 
     # end to end through the public API with host buffers
     e2e = None

@@ -89,7 +89,7 @@ typedef enum {
    * (u, v, zeta) the basis, its derivatives and the rule are products of 1D
    * factors, so the sum over points runs as three short sums, u then v then
    * zeta, over the 13 pairs of separable gradient terms (24 times fewer
-   * flops than the dense contraction at p = 4, 92 times at p = 7).  The same
+   * flops than the dense contraction at p = 4, 112 times at p = 7).  The same
    * kernel as FEI_FP32 at degrees >= 2; degree 1 falls back to FEI_FP32.
    * Output FP32. */
   FEI_SF_FP32 = 4,

@@ -10,8 +10,8 @@
 //   g^_ab[iv][l][iu]  = sum over (m,m') U(m,iu) U(m',iu) X_c[m][m'][iv][l]
 // then the zeta transform's transpose, and per point the step from the
 // collapsed operators to Dt.  Rows are taken in groups of one or two m (Y and X
-// of a group at a time).  It costs what the forward costs: 0.24 MFLOP per
-// element at p = 4, 3.7 at p = 7 (the dense W = gA G^T: 5.7 and 340).
+// of a group at a time).  It costs what the forward costs: 0.23 MFLOP per
+// element at p = 4, 3.0 at p = 7 (the dense W = gA G^T: 5.7 and 340).
 //
 // The Jacobian is recomputed at every point (never stored) and the chain
 // from dL/dDt to the coefficients, to the adjugate rows and det J, to the

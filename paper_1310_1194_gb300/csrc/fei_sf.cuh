@@ -17,7 +17,7 @@
 // other way round), so an entry class (k + k' even or odd) is a thread's
 // work of its own.
 //
-// Per element 0.24 MFLOP at p = 4 and 3.7 MFLOP at p = 7 (the dense
+// Per element 0.23 MFLOP at p = 4 and 3.0 MFLOP at p = 7 (the dense
 // contraction: 5.7 and 340).
 //
 // Blocks are persistent over batches of E elements.  Stages, with one block
@@ -262,8 +262,12 @@ __device__ __forceinline__ void v_zeta_sums(const T *X, const T *fac, int ml, in
   // entry (k, k') of row t; o: A_e[t][t2] (full layout)
   auto store = [&](T *o, int k, int k2, int t, T v) {
     if constexpr (UP) {
-      const int row = k * NT + t, col = k2 * NT + t2;
-      if (col >= row) A[a_pos(row, col, NSH, true)] = v;
+      // column k' NT + t2 >= row k NT + t: every k' > k, none below, and at
+      // k' = k the columns t2 >= t
+      if (k2 > k || (k2 == k && t2 >= t)) {
+        const int row = k * NT + t;
+        A[row * NSH - row * (row + 1) / 2 + k2 * NT + t2] = v;
+      }
     } else {
       o[k * NT * NSH + k2 * NT] = v;
     }
