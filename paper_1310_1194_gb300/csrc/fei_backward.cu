@@ -36,8 +36,9 @@ namespace {
 // thread.  Rows in groups of two m (m = g and M-1-g, alike in size); at p = 7
 // and p = 5 of one m (the shared memory of two and of five blocks per SM; at
 // p = 4 and 6 the further barriers cost more).  GB300, p = 5, 20 000 prisms with
-// per-point fields: 1.27 ms (groups of two m 1.35; 224 threads and 3 blocks
-// 1.6); the dense adjoint on the tensor cores took 5.0.  The parts, by leaving
+// per-point fields: 1.19 ms (gA requested a whole element ahead 1.27, groups of
+// two m 1.35, 224 threads and 3 blocks 1.6); the dense adjoint on the tensor
+// cores took 5.0.  The parts, by leaving
 // them out: zeta sums 0.32 ms (their loads of gA: 0.19 ms of HBM time), v sums
 // 0.16, u sums 0.18, the chain 0.31; the rest is barriers and latency (issue
 // 45 % of slots, 15 to 20 warps an SM).
@@ -52,6 +53,12 @@ struct AdjCfg {
   static constexpr int GM = P == 7 || P == 5 ? 1 : 2, NG = GM == 1 ? M : (M + 1) / 2;
   static constexpr int RM = GM == 1 ? M : M + 1;  // most rows of a group
   static constexpr int NE = (M + 1) / 2, NP = (M + 1) / 2;  // NP: pairs (m', M-1-m')
+  // gA is requested into the L2 one element ahead, or where two elements' gA
+  // of every block would fill it (p = 5: 97 MB of 129, and DRAM reads were
+  // twice gA) one row group ahead.  Forward and adjoint: p = 5, 20 000 prisms
+  // 1.91 -> 1.86 ms, p = 6, 8000 1.67 -> 1.63, p = 7, 4000 1.55 -> 1.37; at p = 4
+  // the whole element is better, 1.76 against 1.80 (40 000)
+  static constexpr bool BY_GROUP = P >= 5;
   // Y [row][t'][l] of 4 values (LL, L'L', LL', L'L); the stride of t' an odd
   // multiple of 4 values against bank conflicts
   static constexpr int YS = 4 * (M % 2 ? M : M + 1);
@@ -69,6 +76,22 @@ struct AdjCfg {
                        Q_LO = Q_G2 + (3 * NQ + 3) / 4 * 4,
                        Q_END = Q_LO + (F32 ? (2 * M * NT + 2 * M * M + 3) / 4 * 4 : 0);
 };
+
+// The rows of gA of row group g on their way to the L2: a point every 128
+// bytes of each row, and its last value.
+template <typename T, int P>
+__device__ __forceinline__ void prefetch_rows(const T *gA, int g, int tid) {
+  using C = AdjCfg<T, P>;
+  constexpr int M = C::M, NT = C::NT, NSH = C::NSH, STEP = 128 / (int)sizeof(T), L = (NSH + STEP - 1) / STEP + 1;
+  const bool single = C::GM == 1 || 2 * g == M - 1;
+  const int n0 = M - g, rows = n0 + (single ? 0 : g + 1);
+  for (int o = tid; o < rows * M * L; o += C::NTH) {
+    const int i = o / L, j = o - i * L, k = i / rows, r = i - k * rows;
+    const int t = r < n0 ? tri_index(g, r) : tri_index(M - 1 - g, r - n0);
+    const T *p = gA + (int64_t)(k * NT + t) * NSH + (j * STEP < NSH - 1 ? j * STEP : NSH - 1);
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+  }
+}
 
 template <typename T, int P>
 struct AdjElem {
@@ -495,12 +518,12 @@ __global__ void __launch_bounds__(AdjCfg<T, P>::NTH, AdjCfg<T, P>::MINB) backwar
     const int64_t aoff = a.A_off ? a.A_off[e] : e * (int64_t)(NSH * NSH);
     const int64_t boff = a.b_off ? a.b_off[e] : e * (int64_t)NSH;
     const int64_t qoff = a.q_off ? a.q_off[e] : e * (int64_t)NQ;
-    // the next element's inputs on their way to the L2 (at p = 7 the gA of
-    // all blocks' next elements would fill it)
+    // the next element's inputs on their way to the L2
+    int64_t anext = -1;
     if (item + gridDim.x < items) {
       const int64_t it = item + gridDim.x, en = a.list ? (int64_t)a.list[it] : it;
-      if (!Q && P <= 6)
-        prefetch_l2(gAg + (a.A_off ? a.A_off[en] : en * (int64_t)(NSH * NSH)), (int)sizeof(T) * NSH * NSH, tid, NTH);
+      anext = a.A_off ? a.A_off[en] : en * (int64_t)(NSH * NSH);
+      if (!Q && !C::BY_GROUP) prefetch_l2(gAg + anext, (int)sizeof(T) * NSH * NSH, tid, NTH);
       if (perq) {
         const int64_t r = a.q_off ? a.q_off[en] : en * (int64_t)NQ;
         prefetch_l2(a.K + 9 * r, 72 * NQ, tid, NTH);
@@ -541,6 +564,10 @@ __global__ void __launch_bounds__(AdjCfg<T, P>::NTH, AdjCfg<T, P>::MINB) backwar
       for (int g = 0; g < C::NG; ++g) {
         const bool single = C::GM == 1 || 2 * g == M - 1;
         const int n0 = M - g, rows = n0 + (single ? 0 : g + 1);
+        if constexpr (C::BY_GROUP) {
+          const bool last = g == C::NG - 1;
+          if (!last || anext >= 0) prefetch_rows<T, P>(gAg + (last ? anext : aoff), last ? 0 : g + 1, tid);
+        }
         // zeta sums: rows of the group, columns t', entry classes
         const int tasks = rows * NT, padded = (tasks + 31) / 32 * 32;
         for (int o = tid; o < 2 * padded; o += NTH) {
