@@ -601,6 +601,8 @@ def run_workload(name, args, ctx, headline):
             dom = {"kernel": "forward", "ms": fwd_ms, "F": F, "precision": precision, "counts": counts,
                    "adjoint_ms": bwd_ms}
     roofline = roofline_of(dom, dom["counts"], dom["precision"], peaks, peak_src, live, Bts, ms, p, n, per_qp)
+    if upper:
+        roofline["traffic"] = None  # the captures are of the full layout
     if plan is not None:
         step_flops = sum(int(counts[d]) * (sf_flops_per_element(d) if runs_sum_factorised(d, prec_of[d]) else
                                            flops_per_element(d)) for d in range(1, 8) if counts[d])

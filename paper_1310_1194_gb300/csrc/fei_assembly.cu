@@ -27,10 +27,11 @@
 //      chunks where a chunk's element matrices would pass a size cap.
 // Device part (fei_assemble): the shared rows are cleared; the entries of
 // private rows (the only contribution they get) are stored by one launch per
-// degree, those of shared rows added by one launch per (degree, colour) run.  fei_integrate_assemble integrates the batch chunk by chunk into one
-// scratch buffer (one forward launch per chunk, all colours of a degree
-// together) and assembles each chunk from it run by run, so that a batch
-// never needs memory for all of its element matrices at once.
+// degree, those of shared rows added by one launch per (degree, colour) run.
+// fei_integrate_assemble integrates the batch chunk by chunk into one scratch
+// buffer (one forward launch per chunk, all colours of a degree together) and
+// assembles each chunk from it run by run, so that a batch never needs memory
+// for all of its element matrices at once.
 #include <stdint.h>
 #include <string.h>
 

@@ -57,8 +57,8 @@ namespace fei {
 //   p = 5,  20 000: 0.68 ms (1.81); R = 2: 0.71, MINB = 6: 0.71
 //   p = 6,  16 384: 1.28 ms (3.8); R = 3: 1.41, MINB = 3: 1.9
 //   p = 7,  16 384: 2.12 ms (6.25); R = 2: 2.26, R = 4: 2.15
-// What bounds it (ncu): issue (p = 4: 71 % of slots, 11.8 k warp instructions
-// an element; p = 7: 56 %, 91 k), with barriers and shared-memory latency as
+// What bounds it (ncu): issue (p = 4: 69 % of slots, 11.5 k warp instructions
+// an element; p = 7: 54 %, 90 k), with barriers and shared-memory latency as
 // the largest stalls; without its stores it takes the same time, DRAM writes
 // are the outputs.  FP64: the FP64 pipe (p = 4, 4096 prisms: 1.25 ms; the
 // dense kernel 23.2 ms).
