@@ -28,7 +28,7 @@
 //   3 the zeta transform of the operators, in place;
 //   then per group of rows (m = g and m = M-1-g: M+1 rows t, so groups are
 //   alike): 4 the u sums into X (one group of X at a time keeps a block's
-//   shared memory small enough for several blocks per SM), 6 the v and zeta
+//   shared memory small enough for several blocks per SM), 5 the v and zeta
 //   sums in registers, with direct stores.
 // In stage 5 a thread owns one column t', up to R rows t of one m, and one
 // entry class.  X is read as 16-byte vectors, each value feeding about six
