@@ -300,7 +300,8 @@ __device__ __forceinline__ void p1_point_contrib(const float *D, const float *G,
 // arithmetic in operations that are rounded one by one (no contraction), so
 // that both kernels give the same bits: 21 FP64 instructions an element
 // instead of about 190 (this part's FP64 rate bound the kernel), at an error
-// of about 2^-44 before the single rounding of w det J.
+// of about 2^-44 before the single rounding of w det J where nothing cancels;
+// the others take FP64 (p1_safe: 1 000 000 prisms 270 -> 274 us).
 __device__ __forceinline__ float2 p1_mul(float2 a, float2 b) {
   const float p = __fmul_rn(a.x, b.x);
   float e = __fmaf_rn(a.x, b.x, -p);
@@ -350,10 +351,41 @@ __device__ __forceinline__ float2 p1_cross_pair(float2 a1, float2 a2, float2 b1,
 // (p_v + p_v+1) + p_v+2
 __device__ __forceinline__ float2 p1_sum3(float2 a, float2 b, float2 c) { return p1_norm(p1_add(p1_add(a, b), c)); }
 
-// The same setup in FP64, for an element with a vertex difference outside
-// 2^-60 <= |d| < 2^60 (other than 0): ev32 [21], then the node sums [2][3]
-// as pairs (12 values).  Not inlined: the compiler would execute its FP64
-// instructions ahead of the branch.
+// Whether the pairs' det J is safe at every point.  The pairs lose what the
+// differences of products in n3 and the sums n3.C, n3.D1, n3.D2 cancel (their
+// error is about 2^-42 of q = sum_k (|c1||c2| terms of n3_k) (|C_k| + |D1_k| +
+// |D2_k|) bounds, which cancel nothing): an element whose det J is not above
+// 2^-14 q at the corners of both node triangles (the points are inside), thin,
+// flat, collapsed or mirrored, or near the ends of the FP32 range, takes the
+// FP64 setup, where n3 of a collapsed triangle is 0.  Rounded operations only,
+// in one order: both p = 1 kernels decide alike.
+__device__ __forceinline__ float p1_gate(const float *ev) {
+  float m1[3], m2[3], md[3], q = 0.f;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    m1[k] = __fadd_rn(fabsf(ev[k]), fabsf(ev[3 + k]));
+    m2[k] = __fadd_rn(fabsf(ev[6 + k]), fabsf(ev[9 + k]));
+    // |v0|, |v1|, |v2| / 2 in terms of C, D1, D2
+    md[k] = __fadd_rn(__fmaf_rn(5.f, fabsf(ev[12 + k]), fabsf(ev[15 + k])), fabsf(ev[18 + k]));
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int i = (k + 1) % 3, j = (k + 2) % 3;
+    q = __fmaf_rn(__fmaf_rn(m1[i], m2[j], __fmul_rn(m1[j], m2[i])), md[k], q);
+  }
+  return __fmul_rn(6.103515625e-5f, q);  // 2^-14 q
+}
+// one vertical node: (a, b, g) = w_z (n3.C, n3.D1, n3.D2)
+__device__ __forceinline__ bool p1_safe(const float2 *zab, float wz, float gate) {
+  const float a = zab[0].x, b = zab[1].x, g = zab[2].x;
+  const float lo = fminf(a, fminf(__fadd_rn(a, b), __fadd_rn(a, g)));
+  return lo > __fmul_rn(wz, gate) && lo > 1e-28f && gate < 1e28f;
+}
+
+// The same setup in FP64, for an element that p1_safe refuses or with a vertex
+// difference outside 2^-60 <= |d| < 2^60 (other than 0): ev32 [21], then the
+// node sums [2][3] as pairs (12 values).  Not inlined: the compiler would
+// execute its FP64 instructions ahead of the branch.
 __device__ __noinline__ void p1_setup64(const double *X, const double *zd, const double *zwd, float *out) {
   double ev[21];
   elem_vectors(X, ev);
@@ -513,6 +545,9 @@ __global__ void __launch_bounds__(kP1Threads, 3) cc_p1_kernel(FwdArgs a) {
           zab[iz][v] = p1_norm(p1_mul(zwp[iz], p1_sum3(p[v], p[(v + 1) % 3], p[(v + 2) % 3])));
         }
       }
+      const float gate = p1_gate(ev32);
+#pragma unroll
+      for (int iz = 0; iz < M; ++iz) in_range &= p1_safe(zab[iz], zwf[iz], gate);
       if (!in_range) {
         float t[33];
         p1_setup64(in, zd, zwd, t);
@@ -733,6 +768,10 @@ __global__ void __launch_bounds__(kP1Threads) cc_p1_small_kernel(FwdArgs a) {
     }
 #pragma unroll
     for (int off = 4; off >= 1; off >>= 1) in_range &= __shfl_xor_sync(0xffffffffu, (int)in_range, off) != 0;
+    // (the same in every lane of the group)
+    const float gate = p1_gate(ev32);
+#pragma unroll
+    for (int n = 0; n < M; ++n) in_range &= p1_safe(zab[n], zwf[n], gate);
     if (!in_range) {
       float t[33];
       p1_setup64(X, zd, zwd, t);

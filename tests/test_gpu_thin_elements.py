@@ -1,0 +1,98 @@
+"""Thin, collapsed and mirrored triangles: n3 = c1 x c2 cancels, so the FP32
+paths must not judge or scale these elements by an FP32 pair's last bits.
+
+The elements: a mesh element moved to the origin (the vertices' rounding
+scales with the element), its third vertices drawn to the line through the
+other two: P2 = P0 + 0.4 (P1 - P0) + eps (P2 - P0), the top alike.  Then c1 x
+c2 is eps times the element's own at every zeta, so det J has the sign of eps
+at every point.  FP64 arithmetic forms w det J to about 10 2^-53 / eps
+(relative), FP32 pairs to at worst 10 2^-44 / eps."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1310_1194_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+KEYS = ("geom", "K", "b", "c", "f")
+NEGATIVE = 3
+
+
+def thin(n, eps):
+    w = inputs.workload("pr1", n_max=max(n, 1))
+    w = {k: np.ascontiguousarray(np.resize(w[k], (n,) + w[k].shape[1:])) for k in KEYS}
+    g = w["geom"] - w["geom"][:, :1]
+    for o in (0, 3):
+        g[:, o + 2] = g[:, o] + 0.4 * (g[:, o + 1] - g[:, o]) + eps * (g[:, o + 2] - g[:, o])
+    w["geom"] = np.ascontiguousarray(g)
+    return w
+
+
+def device(w):
+    return [torch.from_numpy(w[k]).cuda() for k in KEYS]
+
+
+def forward(w, precision, p):
+    from paper_1310_1194_gb300 import api
+    A, b, st, _ = api.fei_integrate(*device(w), p=p, precision=precision)
+    torch.cuda.synchronize()
+    n = len(w["geom"])
+    return A.view(n, -1).double().cpu().numpy(), b.view(n, -1).double().cpu().numpy(), st.cpu().numpy()
+
+
+def rel(x, y):
+    return (np.linalg.norm(x - y, axis=1) / np.linalg.norm(y, axis=1)).max()
+
+
+def check_accuracy(p, precision, n):
+    # FP64 and oracle together: 2 x 10 x 2^-53 / 1e-9 = 2.2e-6, the FP32 path's
+    # own error below 1e-6; its bar is 1e-5
+    w = thin(n, 1e-9)
+    A, b, st = forward(w, precision, p)
+    Ao, bo, so, _ = oracle.integrate(*(w[k] for k in KEYS), p=p)
+    assert not st.any() and not so.any()
+    assert rel(A, Ao.reshape(n, -1)) < 1e-5 and rel(b, bo.reshape(n, -1)) < 1e-5
+
+
+def check_mirrored(p, precision, n):
+    for eps in (-1e-9, -1e-12, -1e-14):
+        A, b, st = forward(thin(n, eps), precision, p)
+        assert (st == NEGATIVE).all(), (eps, int((st != NEGATIVE).sum()))
+        assert not A.any() and not b.any()
+
+
+@pytest.mark.parametrize("n", [3000, 20000])
+def test_p1_thin_and_mirrored(n):
+    """Both p = 1 kernels (one thread per element above 16384)."""
+    check_accuracy(1, "fp32", n)
+    check_mirrored(1, "fp32", n)
+
+
+@pytest.mark.parametrize("n", [3000, 20000])
+def test_p1_collapsed_triangles_are_flagged(n):
+    """P1 == P2 and Q1 == Q2: c1 == c2 at every node, so n3 is 0 exactly."""
+    w = inputs.workload("p1m", n_max=n)
+    w = {k: np.ascontiguousarray(w[k][:n]) for k in KEYS}
+    w["geom"][:, 2] = w["geom"][:, 1]
+    w["geom"][:, 5] = w["geom"][:, 4]
+    A, b, st = forward(w, "fp32", 1)
+    assert (st == NEGATIVE).all(), int((st != NEGATIVE).sum())
+    assert not A.any() and not b.any()
+
+
+def test_p1_kernels_agree_on_thin_elements():
+    """Elements of every kind give the same bits in both kernels."""
+    n, m = 16384 + 300, 300
+    parts = [thin(m, e) for e in (1e-3, 1e-4, 1e-5, 1e-9, 1e-13, -1e-4, -1e-13)]
+    w = inputs.workload("p1m", n_max=n)
+    w = {k: np.ascontiguousarray(w[k][:n]) for k in KEYS}
+    for i, q in enumerate(parts):
+        for k in KEYS:
+            w[k][i::50][:m] = q[k]
+    A, b, st = forward(w, "fp32", 1)
+    As, bs, ss = forward({k: np.ascontiguousarray(w[k][:16000]) for k in KEYS}, "fp32", 1)
+    assert np.array_equal(A[:16000], As) and np.array_equal(b[:16000], bs) and np.array_equal(st[:16000], ss)
+    assert 0 < np.count_nonzero(st) < n
