@@ -52,15 +52,24 @@ struct Elem32 {
   float2 zsum[M][3], zabg[M][3];
   float zc1f[M][3], zc2f[M][3], zn3f[M][3];
   float tc3f[NT][3];
+  float gate;  // w det J above w times this is accurate as a pair (elem_setup32)
 };
 
 // One warp: element vectors (lanes 0-20, component k = j % 3 of vector
-// j / 3) and the vertical-node quantities (lanes 3 iz + k) of the element
-// whose vertices are in el.X.  The vertex differences in FP64 (two
+// v = j / 3) and vertical-node data (lane = 3 iz + k) of one element.  The
+// vertex differences are FP64 subtractions (two per lane, one warp's worth of
 // independent subtractions), split from their bit fields into FP32 pairs,
 // the rest in double-FP32 arithmetic: a dependent FP64 instruction takes
 // hundreds of cycles on this part, an FP32 one a few.  Differences outside
-// 2^-60 <= |d| < 2^60 (other than 0) take the same steps in FP64.
+// 2^-60 <= |d| < 2^60 (other than 0) take the same steps in FP64, and so does
+// an element whose n3 cancels (thin, collapsed or mirrored triangles): the
+// pairs' n3 is good to about 2^-44 of S_k = (|A1| + |B1|) x (|A2| + |B2|) taken
+// with plus signs, so |n3| has to be above 2^-14 of S at every node.
+//
+// gate = 2^-14 q, q = sum_k S_k (5 |C_k| + |D1_k| + |D2_k|) (a bound of the terms
+// of n3 . c3 in which nothing cancels): w det J as a pair has an error of about
+// 2^-42 w q, at most 2^-28 of a value above w gate.  (p = 4, 100 000 prisms: 1.356
+// -> 1.368 ms with these checks.)
 template <int P>
 __device__ __noinline__ void elem_setup32(Elem32<P> &el, const NodeTab32<P> &tb, int lane) {
   constexpr int NZ = P + 1;
@@ -86,46 +95,74 @@ __device__ __noinline__ void elem_setup32(Elem32<P> &el, const NodeTab32<P> &tb,
   const double t1 = xa - xb, t2 = xc - xd;
   bool r1 = true, r2 = true;
   const float2 t1s = split_f64_bits(t1, &r1), t2s = split_f64_bits(t2, &r2);
-  if (__all_sync(0xffffffffu, lane >= 21 || (r1 && r2))) {
+  // gate and whether n3 cancels, from the lane's component of A1, B1, A2, B2,
+  // C, D1, D2 and of n3
+  auto judge = [&](float a1, float b1, float a2, float b2, float c, float d1, float d2, float n3, float *gate) {
+    auto from = [](float v, int src) { return __shfl_sync(0xffffffffu, v, src); };
+    const float m1 = fabsf(a1) + fabsf(b1), m2 = fabsf(a2) + fabsf(b2);
+    const float S = from(m1, l1) * from(m2, l2) + from(m1, l2) * from(m2, l1);
+    const float qk = S * (5.f * fabsf(c) + fabsf(d1) + fabsf(d2)), n = fabsf(n3);
+    const float St = S + from(S, l1) + from(S, l2), nt = n + from(n, l1) + from(n, l2);
+    const float q = qk + from(qk, l1) + from(qk, l2);
+    *gate = q < 1e30f ? 6.103515625e-5f * q : __int_as_float(0x7f800000);  // 2^-14; infinity: always FP64
+    return __any_sync(0xffffffffu, act && !(nt > 6.103515625e-5f * St));
+  };
+  bool pairs = __all_sync(0xffffffffu, lane >= 21 || (r1 && r2));
+  if (pairs) {
     auto shfl2 = [](float2 q, int src) {
       return make_float2(__shfl_sync(0xffffffffu, q.x, src), __shfl_sync(0xffffffffu, q.y, src));
     };
     float2 ev = norm_ff(add_ff(t1s, subtract ? neg_ff(t2s) : t2s));
     ev = make_float2(0.5f * ev.x, 0.5f * ev.y);
     const float2 z2 = tb.ztab2[iz][0], wz2 = tb.ztab2[iz][1];
-    const float2 c1 = norm_ff(add_ff(shfl2(ev, k), mul_ff(z2, shfl2(ev, 3 + k))));
-    const float2 c2 = norm_ff(add_ff(shfl2(ev, 6 + k), mul_ff(z2, shfl2(ev, 9 + k))));
+    const float2 a1 = shfl2(ev, k), b1 = shfl2(ev, 3 + k), a2 = shfl2(ev, 6 + k), b2 = shfl2(ev, 9 + k);
+    const float2 vc = shfl2(ev, 12 + k), vd1 = shfl2(ev, 15 + k), vd2 = shfl2(ev, 18 + k);
+    const float2 c1 = norm_ff(add_ff(a1, mul_ff(z2, b1)));
+    const float2 c2 = norm_ff(add_ff(a2, mul_ff(z2, b2)));
     const float2 c1a = shfl2(c1, l1), c1b = shfl2(c1, l2), c2a = shfl2(c2, l1), c2b = shfl2(c2, l2);
     const float2 n3 = norm_ff(add_ff(mul_ff(c1a, c2b), neg_ff(mul_ff(c1b, c2a))));
-    float2 ab = mul_ff(n3, shfl2(ev, 12 + k));
-    float2 bb = mul_ff(n3, shfl2(ev, 15 + k));
-    float2 gb = mul_ff(n3, shfl2(ev, 18 + k));
+    float2 ab = mul_ff(n3, vc);
+    float2 bb = mul_ff(n3, vd1);
+    float2 gb = mul_ff(n3, vd2);
     ab = norm_ff(add_ff(ab, add_ff(shfl2(ab, l1), shfl2(ab, l2))));
     bb = norm_ff(add_ff(bb, add_ff(shfl2(bb, l1), shfl2(bb, l2))));
     gb = norm_ff(add_ff(gb, add_ff(shfl2(gb, l1), shfl2(gb, l2))));
-    if (lane < 21) el.ev2[lane] = ev;
-    if (act) {
-      const float2 sk = k == 0 ? ab : k == 1 ? bb : gb;
-      el.zsum[iz][k] = sk;
-      el.zabg[iz][k] = norm_ff(mul_ff(wz2, sk));
-      el.zc1f[iz][k] = c1.x;
-      el.zc2f[iz][k] = c2.x;
-      el.zn3f[iz][k] = n3.x;
+    float gate;
+    pairs = !judge(a1.x, b1.x, a2.x, b2.x, vc.x, vd1.x, vd2.x, n3.x, &gate);
+    if (pairs) {
+      if (lane == 0) el.gate = gate;
+      if (lane < 21) el.ev2[lane] = ev;
+      if (act) {
+        const float2 sk = k == 0 ? ab : k == 1 ? bb : gb;
+        el.zsum[iz][k] = sk;
+        el.zabg[iz][k] = norm_ff(mul_ff(wz2, sk));
+        el.zc1f[iz][k] = c1.x;
+        el.zc2f[iz][k] = c2.x;
+        el.zn3f[iz][k] = n3.x;
+      }
     }
-  } else {
+  }
+  if (!pairs) {
     const double ev = 0.5 * (subtract ? t1 - t2 : t1 + t2);
     const double z = tb.zz[iz], wz = tb.zw[iz];
-    const double c1 = fma(z, __shfl_sync(0xffffffffu, ev, 3 + k), __shfl_sync(0xffffffffu, ev, k));
-    const double c2 = fma(z, __shfl_sync(0xffffffffu, ev, 9 + k), __shfl_sync(0xffffffffu, ev, 6 + k));
+    const double a1 = __shfl_sync(0xffffffffu, ev, k), b1 = __shfl_sync(0xffffffffu, ev, 3 + k);
+    const double a2 = __shfl_sync(0xffffffffu, ev, 6 + k), b2 = __shfl_sync(0xffffffffu, ev, 9 + k);
+    const double vc = __shfl_sync(0xffffffffu, ev, 12 + k), vd1 = __shfl_sync(0xffffffffu, ev, 15 + k);
+    const double vd2 = __shfl_sync(0xffffffffu, ev, 18 + k);
+    const double c1 = fma(z, b1, a1);
+    const double c2 = fma(z, b2, a2);
     const double c1a = __shfl_sync(0xffffffffu, c1, l1), c1b = __shfl_sync(0xffffffffu, c1, l2);
     const double c2a = __shfl_sync(0xffffffffu, c2, l1), c2b = __shfl_sync(0xffffffffu, c2, l2);
     const double n3 = c1a * c2b - c1b * c2a;
-    double ab = n3 * __shfl_sync(0xffffffffu, ev, 12 + k);
-    double bb = n3 * __shfl_sync(0xffffffffu, ev, 15 + k);
-    double gb = n3 * __shfl_sync(0xffffffffu, ev, 18 + k);
+    double ab = n3 * vc;
+    double bb = n3 * vd1;
+    double gb = n3 * vd2;
     ab += __shfl_sync(0xffffffffu, ab, l1) + __shfl_sync(0xffffffffu, ab, l2);
     bb += __shfl_sync(0xffffffffu, bb, l1) + __shfl_sync(0xffffffffu, bb, l2);
     gb += __shfl_sync(0xffffffffu, gb, l1) + __shfl_sync(0xffffffffu, gb, l2);
+    float gate;
+    judge((float)a1, (float)b1, (float)a2, (float)b2, (float)vc, (float)vd1, (float)vd2, (float)n3, &gate);
+    if (lane == 0) el.gate = gate;
     if (lane < 21) el.ev2[lane] = split_f64(ev);
     if (act) {
       const double sk = k == 0 ? ab : k == 1 ? bb : gb;
@@ -168,35 +205,31 @@ __device__ __forceinline__ void t_column_from_vertices(const double *X, double x
   }
 }
 
-// w det J at vertical node iz and triangle node t in FP64, from the vertices.
+// det J at vertical node iz and triangle node t in FP64, from the vertices.
 template <int P>
-__device__ __noinline__ double point_wdet64(const Elem32<P> &el, const NodeTab32<P> &tb, int iz, int t,
-                                            const double *tnode) {
+__device__ __noinline__ double point_det64(const Elem32<P> &el, const NodeTab32<P> &tb, int iz, int t,
+                                           const double *tnode) {
   double c1[3], c2[3], n3[3], c3[3];
   z_columns_from_vertices(el.X, tb.zz[iz], c1, c2, n3);
   t_column_from_vertices(el.X, tnode[4 * t], tnode[4 * t + 1], c3);
-  const double wz = tb.zw[iz], wt = tnode[4 * t + 2];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) n3[k] *= wz, c3[k] *= wt;
   return dot3(n3, c3);
 }
 
 // w det J at vertical node iz and triangle node t, rounded once to FP32, and
-// the point's status.  w det J = w_t (a + xi1 b + xi2 g) from the node sums
-// in double-FP32; a value that is not clearly positive against its own terms
-// (2^-13 of them, far above the pairs' 2^-44), or near the ends of the FP32
-// range, is formed again in FP64 from the vertices, so that the status
-// always is that of the FP64 value.
+// the point's status; w: the point's weight.  w det J = w_t (a + xi1 b + xi2 g)
+// from the node sums in double-FP32; a value that is not above w times the
+// element's gate (elem_setup32), or near the lower end of the FP32 range, is
+// formed again in FP64 from the vertices, so that a value that an FP32 pair
+// could get wrong, in sign or in its FP32 digits, is an FP64 one.
 template <int P>
-__device__ __forceinline__ float point_wdet32(const Elem32<P> &el, const NodeTab32<P> &tb, int iz, int t,
+__device__ __forceinline__ float point_wdet32(const Elem32<P> &el, const NodeTab32<P> &tb, int iz, int t, float w,
                                               const double *tnode, int *status) {
-  const float2 pa = mul_ff(tb.ttab2[t][0], el.zabg[iz][0]), pb = mul_ff(tb.ttab2[t][1], el.zabg[iz][1]),
-               pg = mul_ff(tb.ttab2[t][2], el.zabg[iz][2]);
-  const float2 sd = add_ff(add_ff(pa, pb), pg);
-  const float s = sd.x + sd.y, scale = fabsf(pa.x) + fabsf(pb.x) + fabsf(pg.x);
+  const float2 sd = add_ff(add_ff(mul_ff(tb.ttab2[t][0], el.zabg[iz][0]), mul_ff(tb.ttab2[t][1], el.zabg[iz][1])),
+                           mul_ff(tb.ttab2[t][2], el.zabg[iz][2]));
+  const float s = sd.x + sd.y;
   *status = 0;
-  if (s > 1.220703125e-4f * scale && s > 1e-30f && scale < 1e30f) return s;
-  const double sw = point_wdet64<P>(el, tb, iz, t, tnode);
+  if (s > w * el.gate && s > 1e-30f) return s;
+  const double sw = tb.zw[iz] * tnode[4 * t + 2] * point_det64<P>(el, tb, iz, t, tnode);
   // p = 2: a value outside the FP32 range is flagged as well
   *status = point_status(P <= 2 ? (double)(float)sw : sw);
   return (float)sw;

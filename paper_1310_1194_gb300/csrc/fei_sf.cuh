@@ -564,9 +564,9 @@ __global__ void __launch_bounds__(SfCfg<T, P>::NTH, SfCfg<T, P>::MINB) sf_forwar
       T a0[3], a1[3], a2[3], Dq[16], s, w;
       if constexpr (F32) {
         int st;
-        s = point_wdet32<P>(S.el, nodes, iz, t, a.tnode, &st);
-        pst = merge_status(pst, st);
         w = nodes.zwf[iz] * nodes.twf[t];
+        s = point_wdet32<P>(S.el, nodes, iz, t, w, a.tnode, &st);
+        pst = merge_status(pst, st);
         cross3(S.el.zc2f[iz], S.el.tc3f[t], a0);
         cross3(S.el.tc3f[t], S.el.zc1f[iz], a1);
 #pragma unroll

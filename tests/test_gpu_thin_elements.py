@@ -21,12 +21,12 @@ KEYS = ("geom", "K", "b", "c", "f")
 NEGATIVE = 3
 
 
-def thin(n, eps):
+def thin(n, eps, at=0.4):
     w = inputs.workload("pr1", n_max=max(n, 1))
     w = {k: np.ascontiguousarray(np.resize(w[k], (n,) + w[k].shape[1:])) for k in KEYS}
     g = w["geom"] - w["geom"][:, :1]
     for o in (0, 3):
-        g[:, o + 2] = g[:, o] + 0.4 * (g[:, o + 1] - g[:, o]) + eps * (g[:, o + 2] - g[:, o])
+        g[:, o + 2] = g[:, o] + at * (g[:, o + 1] - g[:, o]) + eps * (g[:, o + 2] - g[:, o])
     w["geom"] = np.ascontiguousarray(g)
     return w
 
@@ -96,3 +96,53 @@ def test_p1_kernels_agree_on_thin_elements():
     As, bs, ss = forward({k: np.ascontiguousarray(w[k][:16000]) for k in KEYS}, "fp32", 1)
     assert np.array_equal(A[:16000], As) and np.array_equal(b[:16000], bs) and np.array_equal(st[:16000], ss)
     assert 0 < np.count_nonzero(st) < n
+
+
+SAMPLE = {2: 2000, 3: 600, 4: 300, 5: 100, 6: 60, 7: 40}  # the oracle's share: seconds
+
+
+def fractions(n):
+    return np.random.default_rng(7).uniform(0.1, 0.9, (n, 1))
+
+
+@pytest.mark.parametrize("precision", ["fp32", "sf_fp32"])
+@pytest.mark.parametrize("p", range(2, 8))
+def test_thin_accuracy(p, precision):
+    """eps = 1e-10, the foot of the height anywhere on the edge.  An FP64 n3
+    has at most 3 roundings of two products of size al |c1|^2 where n3 is
+    eps |c1| |v| sin: 6 x 2^-53 / eps = 0.7e-5, say 1e-5 at 1e-10, in the path and
+    in the oracle; doubled.  FP32 pairs: 2^-44 in the place of 2^-53."""
+    n = SAMPLE[p]
+    w = thin(n, 1e-10, fractions(n))
+    A, b, st = forward(w, precision, p)
+    Ao, bo, so, _ = oracle.integrate(*(w[k] for k in KEYS), p=p)
+    assert not st.any() and not so.any()
+    assert rel(A, Ao.reshape(n, -1)) < 4e-5 and rel(b, bo.reshape(n, -1)) < 4e-5
+
+
+@pytest.mark.parametrize("p,n", [(2, 60000), (3, 20000)])
+def test_thin_mirrored_at_the_end_of_the_pairs(p, n):
+    """-5e-15: above FP64's rounding (1e-15 by the bound above), below a pair's."""
+    A, b, st = forward(thin(n, -5e-15, fractions(n)), "fp32", p)
+    assert (st == NEGATIVE).all(), int((st != NEGATIVE).sum())
+    assert not A.any() and not b.any()
+
+
+@pytest.mark.parametrize("p", range(2, 8))
+def test_thin_mirrored(p):
+    check_mirrored(p, "fp32", {2: 6000, 3: 5000, 4: 4000, 5: 2000, 6: 1000, 7: 500}[p])
+
+
+@pytest.mark.parametrize("p", [2, 5])
+def test_thin_elements_do_not_depend_on_their_neighbours(p):
+    """Elements that take the FP64 setup between elements that do not."""
+    n = 700
+    w = inputs.workload("p4", n_max=n)
+    w = {k: np.ascontiguousarray(w[k][:n]) for k in KEYS}
+    alone, _, _ = forward(w, "fp32", p)
+    parts = thin(n, 1e-9)
+    both = {k: np.ascontiguousarray(np.stack([w[k], parts[k]], 1).reshape((2 * n,) + w[k].shape[1:])) for k in KEYS}
+    A, _, st = forward(both, "fp32", p)
+    assert not st.any() and np.array_equal(A[::2], alone)
+    At, _, _ = forward(parts, "fp32", p)
+    assert np.array_equal(A[1::2], At)
