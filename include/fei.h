@@ -68,7 +68,8 @@ typedef enum {
    * >= 2 (see FEI_SF_FP32), the double loop at degree 1. */
   FEI_FP64 = 0,
   /* Vertex differences in FP64, element vectors and w det J in double-FP32
-   * (rounded once), FP32 point operator and sums on the CUDA cores: sum
+   * (rounded once; in FP64 where their terms cancel: thin, flat, collapsed or
+   * mirrored elements), FP32 point operator and sums on the CUDA cores: sum
    * factorisation at degrees >= 2, the double loop at degree 1.  Output
    * FP32. */
   FEI_FP32 = 1,
@@ -219,8 +220,8 @@ fei_status fei_integrate(const fei_reference_t *refs, int nrefs,
  * Jacobians are recomputed, not stored.  The contraction is the transpose of
  * the sum-factorised forward (see FEI_SF_FP32) at every degree.  Precision:
  * FEI_FP64 (all FP64); every other precision runs the FP32 adjoint (FP32
- * sums and chain, w det J and det J in double-FP32 rounded once, the sums
- * over points as FP32 pairs), with gA and gb in FP32.  No scratch memory but
+ * sums and chain, w det J, det J and the status as FEI_FP32's forward, the
+ * sums over points as FP32 pairs), with gA and gb in FP32.  No scratch memory but
  * the bucketing workspace of a degree array.
  * Elements with a nonzero elem_status from the forward get zero gradients
  * (this call recomputes the status itself).  batch->a_layout must be

@@ -763,12 +763,12 @@ __global__ void __launch_bounds__(AdjCfg<T, P>::NTH, AdjCfg<T, P>::MINB) backwar
       __syncthreads();
     }
 
+    int pst = 0;
     // the chain, one thread per point; acc: 21 element-vector gradients,
     // 11 coefficient gradients, then 3 more (per-element coefficients)
     T acc[36];
 #pragma unroll
     for (int k = 0; k < 36; ++k) acc[k] = T(0);
-    int pst = 0;
 #pragma unroll 1
     for (int q = tid; q < NQ; q += NTH) {
       const int iz = q / NT2, t = q - iz * NT2, iv = t / M, iu = t - iv * M;
@@ -781,17 +781,11 @@ __global__ void __launch_bounds__(AdjCfg<T, P>::NTH, AdjCfg<T, P>::MINB) backwar
       }
       T w, s, det, adj[3][3], cx1[3], cx2[3], cx3[3], z, x1, x2;
       if constexpr (F32) {
-        // w, w det J and det J as FP32 pairs, rounded once
-        const float2 wp = mul_ff(nodes.ztab2[iz][1], nodes.ttab2[t][0]);
+        const float2 wp = mul_ff(nodes.ztab2[iz][1], nodes.ttab2[t][0]);  // rounded once
         w = wp.x + wp.y;
-        const float2 sd =
-            add_ff(add_ff(mul_ff(nodes.ttab2[t][0], E.el.zabg[iz][0]), mul_ff(nodes.ttab2[t][1], E.el.zabg[iz][1])),
-                   mul_ff(nodes.ttab2[t][2], E.el.zabg[iz][2]));
-        s = sd.x + sd.y;
-        const float2 dd = add_ff(add_ff(E.el.zsum[iz][0], mul_ff(nodes.txi2[t][0], E.el.zsum[iz][1])),
-                                 mul_ff(nodes.txi2[t][1], E.el.zsum[iz][2]));
-        det = dd.x + dd.y;
-        pst = merge_status(pst, point_status_f(s));
+        int st;
+        s = point_wdet32<P>(E.el, nodes, iz, t, nodes.zwf[iz] * nodes.twf[t], a.tnode, &st, &det);
+        pst = merge_status(pst, merge_status(st, point_status_f(s)));
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
           cx1[k] = E.el.zc1f[iz][k];

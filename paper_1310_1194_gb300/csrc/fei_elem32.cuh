@@ -220,18 +220,27 @@ __device__ __noinline__ double point_det64(const Elem32<P> &el, const NodeTab32<
 // from the node sums in double-FP32; a value that is not above w times the
 // element's gate (elem_setup32), or near the lower end of the FP32 range, is
 // formed again in FP64 from the vertices, so that a value that an FP32 pair
-// could get wrong, in sign or in its FP32 digits, is an FP64 one.
+// could get wrong, in sign or in its FP32 digits, is an FP64 one.  With det: det J
+// too (the adjoint's, with the forward's status).
 template <int P>
 __device__ __forceinline__ float point_wdet32(const Elem32<P> &el, const NodeTab32<P> &tb, int iz, int t, float w,
-                                              const double *tnode, int *status) {
+                                              const double *tnode, int *status, float *det = nullptr) {
   const float2 sd = add_ff(add_ff(mul_ff(tb.ttab2[t][0], el.zabg[iz][0]), mul_ff(tb.ttab2[t][1], el.zabg[iz][1])),
                            mul_ff(tb.ttab2[t][2], el.zabg[iz][2]));
   const float s = sd.x + sd.y;
   *status = 0;
-  if (s > w * el.gate && s > 1e-30f) return s;
-  const double sw = tb.zw[iz] * tnode[4 * t + 2] * point_det64<P>(el, tb, iz, t, tnode);
+  if (s > w * el.gate && s > 1e-30f) {
+    if (det) {
+      const float2 dd = add_ff(add_ff(el.zsum[iz][0], mul_ff(tb.txi2[t][0], el.zsum[iz][1])),
+                               mul_ff(tb.txi2[t][1], el.zsum[iz][2]));
+      *det = dd.x + dd.y;
+    }
+    return s;
+  }
+  const double d = point_det64<P>(el, tb, iz, t, tnode), sw = tb.zw[iz] * tnode[4 * t + 2] * d;
   // p = 2: a value outside the FP32 range is flagged as well
   *status = point_status(P <= 2 ? (double)(float)sw : sw);
+  if (det) *det = (float)d;
   return (float)sw;
 }
 

@@ -146,3 +146,50 @@ def test_thin_elements_do_not_depend_on_their_neighbours(p):
     assert not st.any() and np.array_equal(A[::2], alone)
     At, _, _ = forward(parts, "fp32", p)
     assert np.array_equal(A[1::2], At)
+
+
+def adjoints(w, p, precision):
+    """Both adjoints on a load of the constant function: dL/df is +- its value
+    times the sum of w det J, in which nothing cancels."""
+    from paper_1310_1194_gb300 import api
+    g, n, s = device(w), len(w["geom"]), api.nsh(p)
+    dt = torch.float64 if precision == "fp64" else torch.float32
+    gA, gb = torch.zeros(n * s * s, dtype=dt, device="cuda"), torch.zeros(n, s, dtype=dt, device="cuda")
+    gb[:, 0] = 1.0
+    general = api.fei_integrate_backward(*g, gA, gb.reshape(-1), p=p, precision=precision)
+    u = torch.zeros(n, s, dtype=torch.float64, device="cuda")
+    u[:, 0] = 1.0
+    return general, api.fei_integrate_backward_quadratic(*g, u.reshape(-1), p=p, precision=precision)
+
+
+def flat(n, eps):
+    """Oblique flat elements: regular triangles, the vertical edge in their plane
+    up to eps of its normal part, so that n3 . c3 cancels and n3 does not."""
+    w = thin(n, 1.0)
+    g = w["geom"]
+    at = np.random.default_rng(8).uniform(0.2, 0.8, (2, n, 1))
+    edge = at[0] * (g[:, 1] - g[:, 0]) + at[1] * (g[:, 2] - g[:, 0]) + eps * (g[:, 3] - g[:, 0])
+    g[:, 3:] = g[:, :3] + edge[:, None]
+    return w
+
+
+MANY = {1: 60000, 2: 60000, 3: 20000, 4: 5000, 5: 500, 6: 500, 7: 500}
+
+
+@pytest.mark.parametrize("kind", ["thin", "flat"])
+@pytest.mark.parametrize("p", range(1, 8))
+def test_adjoint_of_thin_and_flat_elements(p, kind):
+    """The FP32 adjoints against the FP64 ones (the bound of test_thin_accuracy:
+    the three products of n3 . c3 round as the two of n3 do), and zero gradients
+    where the forward flags an element."""
+    def make(n, eps):
+        return thin(n, eps, fractions(n)) if kind == "thin" else flat(n, eps)
+    w = make({1: 2000, **SAMPLE}[p], 1e-10)
+    for got, want in zip(adjoints(w, p, "fp32"), adjoints(w, p, "fp64")):
+        assert float(((got[4] - want[4]).abs() / want[4].abs()).max()) < 4e-5
+    n = MANY[p]
+    w = make(n, -5e-15)
+    assert (forward(w, "fp32", p)[2] == NEGATIVE).all()
+    for grads in adjoints(w, p, "fp32"):
+        for t in grads:
+            assert not t.any(), int(t.reshape(n, -1).any(1).sum())
