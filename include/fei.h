@@ -300,8 +300,8 @@ fei_status fei_plan_execute(fei_plan_t plan, const fei_batch *batch, void *A_out
  * and keeps the fastest per degree.  Candidates: the tensor-core kernel's
  * warp-role variants (p >= 3 under the tensor-core precisions), the
  * sum-factorised kernel with as many blocks as fit or one per SM (p >= 3
- * under FEI_SF_FP32), both of these under FEI_AUTO, or 2/4/8/16 blocks per
- * SM for the CUDA-core kernels.  Synchronous (waits for the stream). */
+ * under FEI_SF_FP32), both of these under FEI_AUTO, or the default grid and
+ * 2/4/8/16 blocks per SM for the CUDA-core precisions.  Synchronous (waits for the stream). */
 fei_status fei_plan_tune(fei_plan_t plan, const fei_batch *batch, void *A_out,
                          void *b_out, int32_t *elem_status, fei_stream_t stream);
 

@@ -12,20 +12,13 @@
 // pointers and replays it afterwards, so a repeated batch costs one graph
 // launch and no host work per degree.
 //
-// Candidates per degree (what fei_plan_tune times):
-//   tensor-core paths (p >= 3, FEI_TC_F16X3, FEI_TC_3XTF32): the warp-role variants of the
-//     tcgen05 kernel (8 or 16 producer warps), one CTA per SM;
-//   sum-factorised path (p >= 3, FEI_SF_FP32): as many blocks as fit on the
-//     SMs, or one per SM;
-//   FEI_AUTO at p >= 3: both of the above (FEI_TC_F16X3 variants and the
-//     sum-factorised kernel), so the fastest kernel within the 1e-6 bar wins;
-//   CUDA-core paths (FEI_FP64, FEI_FP32, and p <= 2 under the other precisions): the
-//     grid of the grid-stride kernel, 2, 4, 8 or 16 blocks per SM.
+// What fei_plan_tune times per degree: fei_candidates.cuh.
 // Every candidate computes the same quantities; variants differ only in the
 // order of a few FP32 additions (load-vector partial sums), so results stay
 // within the path's tolerance whichever candidate a plan picks.
 #include <string.h>
 
+#include "fei_candidates.cuh"
 #include "fei_internal.cuh"
 
 struct fei_plan {
@@ -78,32 +71,13 @@ bool same_batch(const fei_batch &x, const fei_batch &y) {
          x.a_layout == y.a_layout;
 }
 
-// Candidates of degree p: every tensor-core variant (grid: one CTA per
-// SM), the sum-factorised kernel with as many blocks as fit or one per SM,
-// the CUDA-core kernels with 2, 4, 8 or 16 blocks per SM.
-int n_candidates(fei_precision prec, int p) {
+// Candidates of degree p (at most kMaxCandidates).
+int candidates(fei_precision prec, int p, Candidate *out) {
   fei_precision run;
   const KernelKind k = plan_kernel(prec, p, 0, &run);
-  if (prec == FEI_AUTO && p >= 3) return tc_variant_count(p, FEI_TC_F16X3) + 2;
-  return k == KERNEL_TC ? tc_variant_count(p, run) : k == KERNEL_SF ? 2 : 4;
-}
-
-// Candidate c of degree p as (variant, grid cap).
-void candidate(fei_precision prec, int p, int c, int *variant, int64_t *grid_cap) {
-  fei_precision run;
-  const int ntc = (prec == FEI_AUTO && p >= 3) ? tc_variant_count(p, FEI_TC_F16X3) : 0;
-  const KernelKind k = plan_kernel(prec, p, c, &run);
-  if (k == KERNEL_TC) {
-    *variant = c;
-    *grid_cap = 0;
-  } else if (k == KERNEL_SF) {
-    *variant = ntc;
-    *grid_cap = c == ntc ? 0 : 152;
-  } else {
-    static const int per_sm[4] = {2, 4, 8, 16};
-    *variant = 0;
-    *grid_cap = 152 * per_sm[c];
-  }
+  const bool sf_too = prec == FEI_AUTO && p >= 3;
+  const int ntc = k == KERNEL_TC ? tc_variant_count(p, run) : 0;
+  return ntc + 2 > kMaxCandidates ? 0 : list_candidates(k, ntc, sf_too, out);
 }
 
 void fill_args(FwdArgs &a, const fei_batch *b, const fei_reference *r, void *A, void *bv, int32_t *st) {
@@ -292,10 +266,11 @@ extern "C" fei_status fei_plan_tune(fei_plan_t plan, const fei_batch *batch, voi
   for (int p = 1; p <= kPMax && !st; ++p) {
     if (!plan->by_p[p] || counts[p] == 0) continue;
     float best = 3.0e38f;
-    for (int c = 0; c < n_candidates(plan->prec, p) && !st; ++c) {
-      int variant;
-      int64_t cap;
-      candidate(plan->prec, p, c, &variant, &cap);
+    Candidate cand[kMaxCandidates];
+    const int nc = candidates(plan->prec, p, cand);
+    for (int c = 0; c < nc && !st; ++c) {
+      const int variant = cand[c].variant;
+      const int64_t cap = cand[c].grid_cap;
       // one untimed run, then the best of two timed runs
       float t_best = 3.0e38f;
       for (int rep = 0; rep < 3 && !st; ++rep) {
