@@ -332,8 +332,8 @@ class Plan:
         """Times the candidate kernel shapes of every degree on this batch
         and keeps the fastest.  With a cache file (``cache``, else the
         environment variable FEI_AUTOTUNE_CACHE) holding choices for this GPU
-        model and precision, those are applied instead of timing; otherwise
-        the tuned choices are added to it."""
+        model, precision and kernel revision, those are applied instead of
+        timing; otherwise the tuned choices are added to it."""
         path = cache if cache is not None else os.environ.get("FEI_AUTOTUNE_CACHE")
         if path and os.path.exists(path) and self.load_choices(path):
             return self.execute(geom, K, b, c, f, p, degree, per_qp, layout, out)
@@ -361,12 +361,19 @@ class Plan:
     def set_choice(self, p: int, variant: int, grid_cap: int):
         check(lib.fei_plan_set_choice(self.handle, int(p), int(variant), int(grid_cap)), "fei_plan_set_choice")
 
+    # part of the tuning cache's key: raised when a change of the kernels makes
+    # stored choices stale (a variant or grid that was the fastest of the kernels
+    # of its time; under the first key "auto" kept the tensor-core kernel at
+    # p = 3, 4, which takes twice the time of today's choice)
+    KERNEL_REVISION = 2
+
     def _cache_key(self):
-        return f"{torch.cuda.get_device_name()}|{self.precision}"
+        return f"{torch.cuda.get_device_name()}|{self.precision}|r{self.KERNEL_REVISION}"
 
     def save_choices(self, path: str):
         """The tuning cache: this plan's per-degree choices, added to the
-        JSON file under the key "<GPU model>|<precision>" (other keys kept)."""
+        JSON file under the key "<GPU model>|<precision>|r<kernel revision>"
+        (other keys kept)."""
         import json
         data = {}
         if os.path.exists(path):
@@ -380,8 +387,8 @@ class Plan:
         os.replace(tmp, path)
 
     def load_choices(self, path: str) -> bool:
-        """Applies the choices stored for this GPU model and precision;
-        returns False (and changes nothing) if the file has none."""
+        """Applies the choices stored for this GPU model, precision and kernel
+        revision; returns False (and changes nothing) if the file has none."""
         import json
         with open(path) as fh:
             data = json.load(fh)
