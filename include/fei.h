@@ -98,9 +98,10 @@ typedef enum {
    * the FP64 oracle (relative Frobenius norm per element): the FEI_FP32
    * kernels for p <= 2 and the sum-factorised kernel for p >= 3; on a
    * direct call p = 3, 4 batches of at most 512 elements give the bits of
-   * FEI_TC_F16X3.  A plan starts from the sum-factorised kernel at p >= 3;
-   * its tuner times the tensor-core variants and the sum-factorised kernel
-   * and keeps the fastest.  Output FP32. */
+   * FEI_TC_F16X3.  A plan runs what a direct call of the batch's size runs,
+   * bit for bit, until its tuner has timed the tensor-core variants and the
+   * sum-factorised kernel and keeps the fastest, or a choice is set.  Output
+   * FP32. */
   FEI_AUTO = 5
 } fei_precision;
 
@@ -323,7 +324,8 @@ fei_status fei_plan_set_choice(fei_plan_t plan, int p, int variant, int64_t grid
 
 /* The kernel the plan's current choice runs for degree p (host pointer):
  * 0 the CUDA-core kernels, 1 the tensor-core kernel, 2 the sum-factorised
- * kernel.  Errors: INVALID_ARG (NULL plan or kernel), INVALID_DEGREE. */
+ * kernel (a plan of FEI_AUTO without a choice at p = 3, 4: that of batches of
+ * more than 512 elements).  Errors: INVALID_ARG (NULL plan or kernel), INVALID_DEGREE. */
 fei_status fei_plan_kernel(fei_plan_t plan, int p, int *kernel);
 
 /* Batch-level summary of the per-element statuses (device int32

@@ -31,6 +31,7 @@ struct fei_plan {
   int32_t *lists;   // [7][max_elem]
   int variant[fei::kPMax + 1];
   int64_t grid_cap[fei::kPMax + 1];
+  bool chosen[fei::kPMax + 1];  // by fei_plan_tune or fei_plan_set_choice
   float tuned_ms[fei::kPMax + 1];
   // graph of the last argument set
   bool has_graph;
@@ -61,6 +62,13 @@ int n_variants(fei_precision prec, int p) {
 // The variant a plan starts from (before any tuning).
 int default_variant(fei_precision prec, int p) {
   return (prec == FEI_AUTO && p >= 3) ? tc_variant_count(p, FEI_TC_F16X3) : 0;
+}
+// The variant a batch of n elements runs: the chosen one, or, where none was
+// chosen, what a direct call of n elements runs (FEI_AUTO at p = 3, 4 has two
+// kernels by n), so that an untuned plan gives a direct call's bits.
+int variant_for(const fei_plan *pl, int p, int64_t n) {
+  fei_precision run;
+  return !pl->chosen[p] && direct_kernel(pl->prec, p, n, &run) == KERNEL_TC ? 0 : pl->variant[p];
 }
 
 // The batch a graph was captured for, field by field (not the padding).
@@ -140,13 +148,13 @@ fei_status enqueue_bucketing(const fei_plan *pl, const fei_batch *b, int32_t *st
 fei_status enqueue_all(const fei_plan *pl, const fei_batch *b, void *A, void *bv, int32_t *st, cudaStream_t s) {
   if (!b->degree) {
     const int p = b->uniform_degree;
-    return launch_degree(pl, p, pl->variant[p], pl->grid_cap[p], b, A, bv, st, false, s);
+    return launch_degree(pl, p, variant_for(pl, p, b->n_elem), pl->grid_cap[p], b, A, bv, st, false, s);
   }
   fei_status e = enqueue_bucketing(pl, b, st, s);
   if (e) return e;
   for (int p = 1; p <= kPMax; ++p) {
     if (!pl->by_p[p]) continue;
-    e = launch_degree(pl, p, pl->variant[p], pl->grid_cap[p], b, A, bv, st, true, s);
+    e = launch_degree(pl, p, variant_for(pl, p, b->n_elem), pl->grid_cap[p], b, A, bv, st, true, s);
     if (e) return e;
   }
   return FEI_OK;
@@ -292,6 +300,7 @@ extern "C" fei_status fei_plan_tune(fei_plan_t plan, const fei_batch *batch, voi
         plan->variant[p] = variant;
         plan->grid_cap[p] = cap;
         plan->tuned_ms[p] = t_best;
+        plan->chosen[p] = true;
       }
     }
   }
@@ -376,6 +385,7 @@ extern "C" fei_status fei_plan_set_choice(fei_plan_t plan, int p, int variant, i
   plan->variant[p] = variant;
   plan->grid_cap[p] = grid_cap;
   plan->tuned_ms[p] = -1.f;
+  plan->chosen[p] = true;
   drop_graph(plan);  // the next execute captures with the new choice
   return FEI_OK;
 }
