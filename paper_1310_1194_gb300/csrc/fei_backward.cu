@@ -71,10 +71,11 @@ struct AdjCfg {
   static constexpr int O_GF = O_G2 + (NQ + 3) / 4 * 4;          // [NQ]
   static constexpr int END = O_GF + (NQ + 3) / 4 * 4;
   // quadratic-loss adjoint: the tables, G1 [2][M][NT] (FP32: pairs), G2
-  // [3][NQ], and in FP32 the rounding errors of VC, ZL and ZD
+  // [3][NQ], and in FP32 the rounding errors of VC, of ZL .. SU and of U0, U1
   static constexpr int Q_G1 = SfTab<P>::SIZE, Q_G2 = Q_G1 + (F32 ? 2 : 1) * (O_G2 - O_G1),
                        Q_LO = Q_G2 + (3 * NQ + 3) / 4 * 4,
-                       Q_END = Q_LO + (F32 ? (2 * M * NT + 2 * M * M + 3) / 4 * 4 : 0);
+                       Q_LZ = Q_LO + 2 * M * NT, Q_LU = Q_LZ + 2 * M * M + 2 * M,
+                       Q_END = F32 ? (Q_LU + 2 * M * M + 3) / 4 * 4 : Q_LO;
 };
 
 // The rows of gA of row group g on their way to the L2: a point every 128
@@ -489,10 +490,13 @@ __global__ void __launch_bounds__(AdjCfg<T, P>::NTH, AdjCfg<T, P>::MINB) backwar
   }
   if constexpr (Q && F32) {
     // the factors' rounding errors
-    for (int i = tid; i < 2 * M * NT + 2 * M * M; i += NTH) {
-      const int j = i < 2 * M * NT ? SfTab<P>::O_VC + i : SfTab<P>::O_ZL + i - 2 * M * NT;
-      sm[C::Q_LO + i] = (float)(gtab64[j] - (double)gtab[j]);
-    }
+    auto err = [&](int at, int from, int n) {
+      for (int i = tid; i < n; i += NTH) sm[at + i] = (float)(gtab64[from + i] - (double)gtab[from + i]);
+    };
+    err(C::Q_LO, SfTab<P>::O_VC, 2 * M * NT);
+    err(C::Q_LZ, SfTab<P>::O_ZL, 2 * M * M + 2 * M);
+    err(C::Q_LU, SfTab<P>::O_U0, M * M);
+    err(C::Q_LU + M * M, SfTab<P>::O_U1, M * M);
   }
   const T *gv = sm + SfTab<P>::O_GV, *su = sm + SfTab<P>::O_SU, *u0 = sm + SfTab<P>::O_U0, *u1 = sm + SfTab<P>::O_U1,
           *zl = sm + SfTab<P>::O_ZL, *zd = sm + SfTab<P>::O_ZD;
@@ -702,7 +706,7 @@ __global__ void __launch_bounds__(AdjCfg<T, P>::NTH, AdjCfg<T, P>::MINB) backwar
         // that v_q carries no more rounding than one dense FP32 sum
         float2 *W = reinterpret_cast<float2 *>(G1);
         const float2 *vlo = reinterpret_cast<const float2 *>(sm + C::Q_LO);
-        const float *zlo = sm + C::Q_LO + 2 * M * NT;
+        const float *zlo = sm + C::Q_LZ;
         for (int o = tid; o < M * NT; o += NTH) {
           const int iz = o / NT, t = o - iz * NT;
           float2 p = make_float2(0.f, 0.f), d = p;
@@ -817,6 +821,18 @@ __global__ void __launch_bounds__(AdjCfg<T, P>::NTH, AdjCfg<T, P>::MINB) backwar
       if constexpr (Q) {
         T v0 = T(0), v1 = T(0), v2 = T(0), v3 = T(0);
         const T *p = G2 + (iz * M + iv) * M;
+        if constexpr (F32) {
+          // the factors' rounding errors first: the same for every element and
+          // point, they would not average out of the sums over the points
+          const T *ul = sm + C::Q_LU + iu;
+#pragma unroll
+          for (int m = 0; m < M; ++m) {
+            v0 += ul[m * M] * p[m];
+            v1 += ul[(M + m) * M] * p[m];
+            v2 += ul[m * M] * p[NQ + m];
+            v3 += ul[m * M] * p[2 * NQ + m];
+          }
+        }
 #pragma unroll
         for (int m = 0; m < M; ++m) {
           const T um = u0[m * M + iu];
@@ -825,7 +841,12 @@ __global__ void __launch_bounds__(AdjCfg<T, P>::NTH, AdjCfg<T, P>::MINB) backwar
           v2 += um * p[NQ + m];
           v3 += um * p[2 * NQ + m];
         }
-        v1 *= gp;
+        if constexpr (F32) {
+          v1 = fmaf(gp, v1, sm[C::Q_LZ + 2 * M * M + iv] * v1);
+          v2 += sm[C::Q_LZ + 2 * M * M + M + iu] * v1;
+        } else {
+          v1 *= gp;
+        }
         v2 += sp * v1;
         const T v[3] = {v1, v2, v3};
         gD00 = v0 * v0;
