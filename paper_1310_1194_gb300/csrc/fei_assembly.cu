@@ -61,7 +61,7 @@ struct fei_assembly {
   std::vector<int64_t> run_start;  // runs of equal (degree, colour) in elems: [runs + 1]
   std::vector<int32_t> run_degree;  // [runs]
   struct Chunk {
-    int32_t colour, degree;
+    int32_t degree;
     int64_t start, n, a_len, b_len;
   };
   std::vector<Chunk> chunks;
@@ -80,12 +80,9 @@ struct fei_assembly {
   int32_t *shrows;   // global rows touched by several elements (cleared first)
   int64_t n_shrows;
   bool has_private[fei::kPMax + 1];  // degrees with rows that one element alone touches
-  int32_t *elems;        // elements sorted by (colour, degree)
+  int32_t *elems;        // elements sorted by (degree, colour)
   int32_t *chunk_count;  // [chunks] element count of each chunk (the forward's device count)
   int64_t *scr_aoff, *scr_boff;  // start of element e in its chunk's scratch
-  // fused path: two scratch buffers (chunk k uses buffer k % 2), the stream
-  // that assembles while the caller's stream integrates the next chunk, and
-  // the events that order the two
   // fused path: the chunk scratch (element matrices and vectors), allocated
   // on first use
   void *scratch_A, *scratch_b;
@@ -438,14 +435,14 @@ fei_status build(fei_assembly *as, const int64_t *l2g) {
   as->chunks.clear();
   as->max_chunk_a = as->max_chunk_b = 0;
   for (int64_t k = 0; k < n;) {
-    const int32_t e0 = elems[k], c = as->colour_h[e0], p = as->degree_h[e0];
+    const int32_t p = as->degree_h[elems[k]];
     const int64_t s = nsh_of(p);
     // all elements of a degree unless their matrices pass the cap (the
     // forward kernels want large launches), and at least a few tiles per SM
     int64_t cap = kChunkBytes / (4 * s * s);
     const int64_t tiles_min = 8ll * 152 * 128 / s;
     if (cap < tiles_min) cap = tiles_min;
-    fei_assembly::Chunk ch{c, p, k, 0, 0, 0};
+    fei_assembly::Chunk ch{p, k, 0, 0, 0};
     while (k < n && ch.n < cap && as->degree_h[elems[k]] == p) {
       scr_aoff[elems[k]] = ch.a_len;
       scr_boff[elems[k]] = ch.b_len;
@@ -670,7 +667,7 @@ extern "C" fei_status fei_integrate_assemble(fei_assembly_t as, const fei_refere
   }
   cudaStream_t s = (cudaStream_t)stream;
   if ((st = clear_outputs(as, vb, values, rhs, s))) return st;
-  // chunk by chunk, in (colour, degree) order: integrate into the scratch,
+  // chunk by chunk, in (degree, colour) order: integrate into the scratch,
   // then assemble from it (the next chunk's forward follows on the stream)
   for (size_t ci = 0; ci < as->chunks.size(); ++ci) {
     const auto &ch = as->chunks[ci];

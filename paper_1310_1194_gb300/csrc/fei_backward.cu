@@ -97,7 +97,6 @@ __device__ __forceinline__ void prefetch_rows(const T *gA, int g, int tid) {
 template <typename T, int P>
 struct AdjElem {
   std::conditional_t<std::is_same<T, float>::value, Elem32<P>, Elem64<P>> el;
-  double cd[14];
   T cf[14];
   int status;
   double gev[21];

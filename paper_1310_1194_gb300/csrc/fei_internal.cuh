@@ -5,8 +5,6 @@
 //   pts   double [N_q][4]        (xi1, xi2, zeta, w)
 //   G64   double [N_q][4][N_sh]  row 0 = phi, rows 1..3 = d phi / d(xi1, xi2, zeta)
 //   G32   float  [N_q][4][N_sh]  the same rounded to FP32
-//   G32T  float  [N_q][N_sh][4]  the same, components adjacent (one 16-byte
-//                                load per point and shape function)
 //   znode double [p+1][2]        (zeta, w_zeta)        vertical Gauss nodes
 //   tnode double [(p+1)^2][4]    (xi1, xi2, w_tri, 0)  collapsed triangle nodes
 //   point q = iz * (p+1)^2 + t, t = iv * (p+1) + iu, w_q = w_tri[t] w_zeta[iz].
@@ -41,7 +39,6 @@ struct fei_reference {
   float *G32;
   double *znode;
   double *tnode;
-  float *G32T;       // [N_q][N_sh][4] the FP32 table with the 4 components adjacent
   fei::TcImage *tc;  // null until built (degree >= 3)
   float *sf;         // 1D factor tables of the sum-factorised paths, or null
   double *sf64;      // the same in FP64
@@ -74,7 +71,6 @@ struct FwdArgs {
   const float *G32;
   const double *znode;
   const double *tnode;
-  const float *G32T;
 };
 
 // Values of one A_e: N_sh^2, or N_sh (N_sh + 1) / 2 in the upper layout.
@@ -164,8 +160,9 @@ fei_status integrate_scratch(const fei_reference *const *by_p, const fei_batch *
                              int32_t *lists, int64_t cap, cudaStream_t s);
 
 // Kernel launchers (each returns FEI_OK or an error already recorded).
-// grid_cap: largest grid (blocks) of the grid-stride kernels, 0 = default
-// (all work items for a known count, 152 x 4 or 152 x 8 for a device count)
+// grid_cap: largest grid (blocks) of the persistent kernels, 0 = default (the
+// blocks that fit on the device, fewer where a known count needs fewer; p = 1:
+// 152 x 3 blocks, FP64 152 x 4 for a device count and one pass for a known one)
 fei_status launch_cc_forward(int p, bool fp64, const fei_reference *ref, const FwdArgs &a, int64_t grid_work,
                              cudaStream_t s, int64_t grid_cap = 0);
 // quadratic = true: the adjoint of L = sum_e u_e^T A_e u_e - u_e^T b_e
@@ -177,18 +174,22 @@ inline bool tc_precision(fei_precision prec) { return prec == FEI_TC_F16X3 || pr
 inline bool valid_precision(fei_precision prec) {
   return prec == FEI_FP64 || prec == FEI_FP32 || tc_precision(prec) || prec == FEI_SF_FP32 || prec == FEI_AUTO;
 }
-// The kernels of the forward: CUDA-core (fei_cc.cu), tensor-core
-// (fei_tc.cu) and sum-factorised (fei_sf.cu).  The tensor-core and
-// sum-factorised kernels run degrees >= 3; lower degrees of those
-// precisions run the FEI_FP32 CUDA-core kernels.
+// The kernels of the forward: the CUDA-core precisions FEI_FP32 and FEI_FP64
+// (fei_cc.cu: p = 1 kernels, the sum-factorised ones above), tensor-core
+// (fei_tc.cu) and sum-factorised (fei_sf.cu, FEI_SF_FP32).  KERNEL_TC and
+// KERNEL_SF are what degrees >= 3 of those precisions run; their lower degrees
+// run FEI_FP32.
 enum KernelKind { KERNEL_CC = 0, KERNEL_TC = 1, KERNEL_SF = 2 };
 // The kernel of degree p under prec on a direct call of n_batch elements, and
 // the precision it runs in (FEI_AUTO resolved per degree).  FEI_AUTO at
-// p = 3, 4 keeps the bits of FEI_TC_F16X3 for small batches, as documented;
-// above kAutoTcMax it runs the sum-factorised kernel, the faster of the two
-// (GB300, p = 4: 1000 prisms 23 against 40 us, 100 000 prisms 1.58 against
-// 2.81 ms; p = 3: 1000 prisms 14 against 23 us) and the closer one to FP64
-// (1.6e-7 against 4.1e-7).
+// p = 3, 4: the sum-factorised kernel is the faster at every size and the closer
+// one to FP64 (1.6e-7 against 4.1e-7).  Up to kAutoTcMax elements FEI_AUTO all the
+// same gives the bits of FEI_TC_F16X3, as documented for direct calls (fei.h), so
+// that small reference results of callers stay what they were; the line is not a
+// crossing point.  GB300, one call, tensor-core / sum-factorised, us:
+//   p = 3: 1 element 26 / 24, 300 27 / 25, 512 32 / 27, 1000 37 / 28, 3000 59 / 37
+//   p = 4: 1 element 33 / 27, 300 40 / 30, 512 39 / 31, 1000 54 / 37, 3000 114 / 64
+//   (100 000 at p = 4: 2.81 / 1.37 ms)
 constexpr int64_t kAutoTcMax = 512;
 inline KernelKind direct_kernel(fei_precision prec, int p, int64_t n_batch, fei_precision *run) {
   if (prec == FEI_AUTO)

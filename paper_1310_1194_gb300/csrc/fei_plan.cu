@@ -4,7 +4,7 @@
 // Elements of one degree share the reference tables (Sec. 2.2: elements
 // are grouped by type and degree so that the tables stay in fast memory),
 // so a mixed batch runs as: clear the bucket counts, bucket the elements by
-// degree (one atomic per element), then one persistent kernel per degree
+// degree (one atomic per warp and degree), then one persistent kernel per degree
 // that walks its bucket.  A plan owns the bucket scratch (allocated once, at
 // creation) and, per degree, the kernel variant and grid that its
 // autotuner measured fastest on a real batch.  fei_plan_execute captures the
@@ -109,7 +109,6 @@ void fill_args(FwdArgs &a, const fei_batch *b, const fei_reference *r, void *A, 
   a.G32 = r->G32;
   a.znode = r->znode;
   a.tnode = r->tnode;
-  a.G32T = r->G32T;
 }
 
 fei_status launch_degree(const fei_plan *pl, int p, int variant, int64_t grid_cap, const fei_batch *b, void *A,
