@@ -191,3 +191,29 @@ def test_p1_kernels_agree_in_and_out_of_the_pair_range():
     at = np.r_[0, np.cumsum(np.where(degree == 1, 36, 324))]
     got = np.stack([Al[at[2 * i + 1]:at[2 * i + 2]] for i in range(m)])
     assert np.array_equal(got, A.reshape(n, 36)[:m])
+
+
+@pytest.mark.parametrize("p,per_qp", [(3, False), (4, False), (5, True)])
+def test_adjoint_wide_cotangents_past_the_resident_blocks(p, per_qp):
+    """Cotangents whose rows differ by six orders of magnitude, on about twice
+    as many elements as there are resident blocks: the loop reuses Y, X and D
+    and takes the next element's rows; sampled elements against the oracle
+    (the FP32 adjoint's bars)."""
+    from paper_1310_1194_gb300 import api
+    from parity_util import assert_grads_close
+    n, s, q = {3: 4001, 4: 2003, 5: 1601}[p], api.nsh(p), api.nq(p)
+    w = inputs.workload("diff" if per_qp else "p4", n_max=n)
+    n = len(w["geom"])
+    rng = np.random.default_rng(40 + p)
+    gA = (rng.standard_normal((n, s, s)) * 10.0 ** rng.integers(-3, 4, size=(n, s, 1))).astype(np.float32)
+    gb = rng.standard_normal((n, s)).astype(np.float32)
+    dev = [torch.from_numpy(np.ascontiguousarray(w[k])).cuda() for k in ("geom", "K", "b", "c", "f")]
+    got = api.fei_integrate_backward(*dev, torch.from_numpy(gA).cuda(), torch.from_numpy(gb).cuda(), p=p, per_qp=per_qp,
+                                     precision="fp32")
+    idx = np.r_[0, 1, n // 2, n - 903, n - 2, n - 1]
+    rec = (idx[:, None] * q + np.arange(q)).reshape(-1) if per_qp else idx
+    sub = [w["geom"][idx]] + [w[k][rec] for k in ("K", "b", "c", "f")]
+    ref = oracle.integrate_backward(*(np.ascontiguousarray(x) for x in sub), gA[idx].astype(np.float64).reshape(-1),
+                                    gb[idx].astype(np.float64).reshape(-1), p=p, per_qp=per_qp)
+    out = [got[0].cpu().numpy()[idx]] + [t.cpu().numpy()[rec] for t in got[1:]]
+    assert_grads_close(out, ref, len(idx), per_qp, np.full(len(idx), q), 1e-6, 1e-5, where=f"p={p}")
