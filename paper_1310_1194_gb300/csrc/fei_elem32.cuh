@@ -63,13 +63,15 @@ struct Elem32 {
 // hundreds of cycles on this part, an FP32 one a few.  Differences outside
 // 2^-60 <= |d| < 2^60 (other than 0) take the same steps in FP64, and so does
 // an element whose n3 cancels (thin, collapsed or mirrored triangles): the
-// pairs' n3 is good to about 2^-44 of S_k = (|A1| + |B1|) x (|A2| + |B2|) taken
-// with plus signs, so |n3| has to be above 2^-14 of S at every node.
+// pairs' n3 is good to about 2^-44 of the terms T = |c1a c2b| + |c1b c2a| of its
+// components, so at every node a component has to be above 2^-14 of the largest
+// T of all nodes (all: c1 or c2 may cancel at one of them).
 //
-// gate = 2^-14 q, q = sum_k S_k (5 |C_k| + |D1_k| + |D2_k|) (a bound of the terms
-// of n3 . c3 in which nothing cancels): w det J as a pair has an error of about
-// 2^-42 w q, at most 2^-28 of a value above w gate.  (p = 4, 100 000 prisms: 1.356
-// -> 1.368 ms with these checks.)
+// gate = 3 2^-14 q, q the largest T_k (5 |C_k| + |D1_k| + |D2_k|), so that 3 q bounds
+// the terms of n3 . c3 in which nothing cancels: w det J as a pair has an error
+// of about 2^-42 w 3 q, at most 2^-28 of a value above w gate.  One reduction
+// each; with sums over k by shuffles the setup cost 3 % of the forward at p = 3.
+// (p = 4, 100 000 prisms: 1.357 -> 1.364 ms with these checks, by shuffles 1.369.)
 template <int P>
 __device__ __noinline__ void elem_setup32(Elem32<P> &el, const NodeTab32<P> &tb, int lane) {
   constexpr int NZ = P + 1;
@@ -95,17 +97,18 @@ __device__ __noinline__ void elem_setup32(Elem32<P> &el, const NodeTab32<P> &tb,
   const double t1 = xa - xb, t2 = xc - xd;
   bool r1 = true, r2 = true;
   const float2 t1s = split_f64_bits(t1, &r1), t2s = split_f64_bits(t2, &r2);
-  // gate and whether n3 cancels, from the lane's component of A1, B1, A2, B2,
-  // C, D1, D2 and of n3
-  auto judge = [&](float a1, float b1, float a2, float b2, float c, float d1, float d2, float n3, float *gate) {
-    auto from = [](float v, int src) { return __shfl_sync(0xffffffffu, v, src); };
-    const float m1 = fabsf(a1) + fabsf(b1), m2 = fabsf(a2) + fabsf(b2);
-    const float S = from(m1, l1) * from(m2, l2) + from(m1, l2) * from(m2, l1);
-    const float qk = S * (5.f * fabsf(c) + fabsf(d1) + fabsf(d2)), n = fabsf(n3);
-    const float St = S + from(S, l1) + from(S, l2), nt = n + from(n, l1) + from(n, l2);
-    const float q = qk + from(qk, l1) + from(qk, l2);
-    *gate = q < 1e30f ? 6.103515625e-5f * q : __int_as_float(0x7f800000);  // 2^-14; infinity: always FP64
-    return __any_sync(0xffffffffu, act && !(nt > 6.103515625e-5f * St));
+  // gate and whether n3 cancels, from the terms of the lane's component of n3,
+  // its part of (5 |C| + |D1| + |D2|) and the component (values >= 0 order as their
+  // bits, a NaN above them)
+  auto judge = [&](float terms, float vert, float n3, float *gate) {
+    const float T = act ? terms : 0.f;
+    const float tm = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(T)));
+    const float q = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(T * vert)));
+    *gate = q < 3e29f ? 1.8310546875e-4f * q : __int_as_float(0x7f800000);  // infinity: always FP64
+    unsigned ok = __ballot_sync(0xffffffffu, fabsf(n3) > 6.103515625e-5f * tm);
+    ok |= ok >> 1 | ok >> 2;  // bit 3 iz: one of node iz's components
+    constexpr unsigned nodes = 0x249249u & ((1u << 3 * NZ) - 1u);
+    return (ok & nodes) != nodes;
   };
   bool pairs = __all_sync(0xffffffffu, lane >= 21 || (r1 && r2));
   if (pairs) {
@@ -128,7 +131,8 @@ __device__ __noinline__ void elem_setup32(Elem32<P> &el, const NodeTab32<P> &tb,
     bb = norm_ff(add_ff(bb, add_ff(shfl2(bb, l1), shfl2(bb, l2))));
     gb = norm_ff(add_ff(gb, add_ff(shfl2(gb, l1), shfl2(gb, l2))));
     float gate;
-    pairs = !judge(a1.x, b1.x, a2.x, b2.x, vc.x, vd1.x, vd2.x, n3.x, &gate);
+    pairs = !judge(fabsf(c1a.x * c2b.x) + fabsf(c1b.x * c2a.x), 5.f * fabsf(vc.x) + fabsf(vd1.x) + fabsf(vd2.x), n3.x,
+                   &gate);
     if (pairs) {
       if (lane == 0) el.gate = gate;
       if (lane < 21) el.ev2[lane] = ev;
@@ -161,7 +165,7 @@ __device__ __noinline__ void elem_setup32(Elem32<P> &el, const NodeTab32<P> &tb,
     bb += __shfl_sync(0xffffffffu, bb, l1) + __shfl_sync(0xffffffffu, bb, l2);
     gb += __shfl_sync(0xffffffffu, gb, l1) + __shfl_sync(0xffffffffu, gb, l2);
     float gate;
-    judge((float)a1, (float)b1, (float)a2, (float)b2, (float)vc, (float)vd1, (float)vd2, (float)n3, &gate);
+    judge((float)(fabs(c1a * c2b) + fabs(c1b * c2a)), (float)(5.0 * fabs(vc) + fabs(vd1) + fabs(vd2)), (float)n3, &gate);
     if (lane == 0) el.gate = gate;
     if (lane < 21) el.ev2[lane] = split_f64(ev);
     if (act) {
