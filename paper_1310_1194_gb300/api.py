@@ -505,7 +505,7 @@ class Assembly:
     function get different colours) and the scatter map are built on the
     host; ``assemble`` then adds the element matrices colour by colour
     without atomics, and ``integrate_assemble`` integrates and assembles
-    chunk by chunk through an L2-sized scratch.  ``host_only`` builds the
+    chunk by chunk through one scratch buffer.  ``host_only`` builds the
     pattern and colouring without touching a GPU."""
 
     def __init__(self, l2g, n_dof, p=None, degree=None, host_only=False):

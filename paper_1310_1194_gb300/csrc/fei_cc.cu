@@ -7,8 +7,9 @@
 // formed (steps 7-8, fei_geom.cuh), then the double loop over shape
 // functions (steps 9-13).
 //
-// FEI_FP64: everything in FP64.  FEI_FP32: the vertex differences and the
-// vertical-node sums of det J in FP64, w det J at every point in double-FP32
+// FEI_FP64: everything in FP64.  FEI_FP32: the vertex differences in FP64,
+// element vectors, the vertical-node sums of det J and w det J at every point
+// in double-FP32 (the first two in FP64 where they cancel, p1_safe), w det J
 // rounded once; the adjugate rows, the point operator and the contraction in
 // FP32.
 #include <type_traits>

@@ -11,8 +11,9 @@
 // So c1, c2 depend only on the vertical node and c3 only on the triangle
 // node; det J = (c1 x c2) . c3 and J^{-1} has rows
 //   adj_0 = c2 x c3, adj_1 = c3 x c1, adj_2 = c1 x c2, divided by det J.
-// The element vectors are differences of vertex coordinates and are always
-// formed in FP64 (this is where FP32 would lose the most: |x| ~ 1, h ~ 1/50).
+// The element vectors are sums of differences of vertex coordinates; the
+// differences are always FP64 (this is where FP32 would lose the most: |x| ~ 1,
+// h ~ 1/50).
 //
 // Point operator (Eq. (2) with the general weak form): with
 // T = blockdiag(1, J^{-T}) and D = [[c, b^T], [0, K]] (row = test

@@ -10,6 +10,11 @@ the algorithmic work of their elements, F(p) = 8 N_sh^2 N_q + 2 N_sh N_q +
 the case where one process wants the whole batch; it is not part of the
 integration itself.
 
+A shard is a batch of its own: precision "auto" picks its kernel at p = 3, 4
+by the size of the batch it is called with (include/fei.h), so a shard of at
+most 512 elements of a larger batch gives the other kernel's bits there (both
+within 1e-6 of FP64); a precision named outright gives the whole batch's bits.
+
 Pure host logic plus torch.distributed; it works with the gloo backend on
 CPU tensors and with NCCL on CUDA tensors.
 """
