@@ -41,7 +41,8 @@ namespace {
 // cores took 5.0.  The parts, by leaving
 // them out: zeta sums 0.32 ms (their loads of gA: 0.19 ms of HBM time), v sums
 // 0.16, u sums 0.18, the chain 0.31; the rest is barriers and latency (issue
-// 45 % of slots, 15 to 20 warps an SM).
+// 53 % of slots, 20 warps an SM).  Since then the forward's check of w det J:
+// 1.28 -> 1.31 ms by a profiler's (cold) times.
 template <typename T, int P>
 struct AdjCfg {
   static constexpr bool F32 = std::is_same<T, float>::value;

@@ -235,9 +235,9 @@ __global__ void __launch_bounds__(SmallCfg::WPB * 32) cc_small_kernel(FwdArgs a)
 // registers and runs the points in turn.  Records and results pass through
 // shared memory, so that consecutive threads touch consecutive addresses (a
 // thread's own record or matrix is a line of its own in every load and
-// store).  1 000 000 prisms (GB300): 0.275 ms, 1.56 TB/s of inputs and
+// store).  1 000 000 prisms (GB300): 0.277 ms, 1.53 TB/s of inputs and
 // outputs; with FP64 node sums and per-thread loads and stores 0.467 ms.  It
-// is bound by issue (51 % of slots with the 12 warps an SM that the
+// is bound by issue (55 % of slots with the 12 warps an SM that the
 // registers allow); more blocks per SM spill (4: 0.30, 5: 0.38 ms).
 // ---------------------------------------------------------------------------
 constexpr int kP1Threads = 128;

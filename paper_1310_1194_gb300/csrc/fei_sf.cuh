@@ -53,11 +53,12 @@ namespace fei {
 // dense one at p = 2, the one with 21 term pairs above):
 //   p = 2, 200 000 prisms: 0.49 ms (2.51); MINB = 8: 0.54
 //   p = 3,  60 000: 0.31 ms (1.67); R = 2: 0.36
-//   p = 4, 100 000: 1.34 ms (5.41); R = 5: 1.68, MINB = 5: 1.48
+//   p = 4, 100 000: 1.34 ms (5.41); R = 5: 1.68, MINB = 5: 1.48 (both before
+//                   the element setup's checks, which took 1.336 to 1.344)
 //   p = 5,  20 000: 0.68 ms (1.81); R = 2: 0.71, MINB = 6: 0.71
 //   p = 6,  16 384: 1.28 ms (3.8); R = 3: 1.41, MINB = 3: 1.9
 //   p = 7,  16 384: 2.12 ms (6.25); R = 2: 2.26, R = 4: 2.15
-// What bounds it (ncu): issue (p = 4: 69 % of slots, 11.5 k warp instructions
+// What bounds it (ncu): issue (p = 4: 68 % of slots, 11.4 k warp instructions
 // an element; p = 7: 54 %, 90 k), with barriers and shared-memory latency as
 // the largest stalls; without its stores it takes the same time, DRAM writes
 // are the outputs.  FP64: the FP64 pipe (p = 4, 4096 prisms: 1.25 ms; the
