@@ -226,7 +226,7 @@ fei_status fei_integrate(const fei_reference_t *refs, int nrefs,
  * the bucketing workspace of a degree array.
  * Elements with a nonzero elem_status from the forward get zero gradients
  * (this call recomputes the status itself, as the forward of FEI_FP64 or
- * FEI_FP32 does; the tensor-core forward judges det J by FP32 pairs alone, so
+ * FEI_FP32 does; the tensor-core forward takes det J from FP32 pairs alone, so
  * an element whose det J is below about 2^-44 of the terms it is formed from
  * may be flagged there and not here, or the other way round).  batch->a_layout must be
  * FEI_A_FULL (FEI_ERR_UNSUPPORTED otherwise). */

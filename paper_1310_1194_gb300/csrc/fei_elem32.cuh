@@ -100,7 +100,7 @@ __device__ __noinline__ void elem_setup32(Elem32<P> &el, const NodeTab32<P> &tb,
   // gate and whether n3 cancels, from the terms of the lane's component of n3,
   // its part of (5 |C| + |D1| + |D2|) and the component (values >= 0 order as their
   // bits, a NaN above them)
-  auto judge = [&](float terms, float vert, float n3, float *gate) {
+  auto cancels = [&](float terms, float vert, float n3, float *gate) {
     const float T = act ? terms : 0.f;
     const float tm = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(T)));
     const float q = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(T * vert)));
@@ -131,7 +131,7 @@ __device__ __noinline__ void elem_setup32(Elem32<P> &el, const NodeTab32<P> &tb,
     bb = norm_ff(add_ff(bb, add_ff(shfl2(bb, l1), shfl2(bb, l2))));
     gb = norm_ff(add_ff(gb, add_ff(shfl2(gb, l1), shfl2(gb, l2))));
     float gate;
-    pairs = !judge(fabsf(c1a.x * c2b.x) + fabsf(c1b.x * c2a.x), 5.f * fabsf(vc.x) + fabsf(vd1.x) + fabsf(vd2.x), n3.x,
+    pairs = !cancels(fabsf(c1a.x * c2b.x) + fabsf(c1b.x * c2a.x), 5.f * fabsf(vc.x) + fabsf(vd1.x) + fabsf(vd2.x), n3.x,
                    &gate);
     if (pairs) {
       if (lane == 0) el.gate = gate;
@@ -165,7 +165,7 @@ __device__ __noinline__ void elem_setup32(Elem32<P> &el, const NodeTab32<P> &tb,
     bb += __shfl_sync(0xffffffffu, bb, l1) + __shfl_sync(0xffffffffu, bb, l2);
     gb += __shfl_sync(0xffffffffu, gb, l1) + __shfl_sync(0xffffffffu, gb, l2);
     float gate;
-    judge((float)(fabs(c1a * c2b) + fabs(c1b * c2a)), (float)(5.0 * fabs(vc) + fabs(vd1) + fabs(vd2)), (float)n3, &gate);
+    cancels((float)(fabs(c1a * c2b) + fabs(c1b * c2a)), (float)(5.0 * fabs(vc) + fabs(vd1) + fabs(vd2)), (float)n3, &gate);
     if (lane == 0) el.gate = gate;
     if (lane < 21) el.ev2[lane] = split_f64(ev);
     if (act) {

@@ -1,5 +1,5 @@
 """Thin, collapsed and mirrored triangles: n3 = c1 x c2 cancels, so the FP32
-paths must not judge or scale these elements by an FP32 pair's last bits.
+paths must not flag or scale these elements by an FP32 pair's last bits.
 
 The elements: a mesh element moved to the origin (the vertices' rounding
 scales with the element), its third vertices drawn to the line through the
